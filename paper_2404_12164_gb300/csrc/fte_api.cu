@@ -265,16 +265,16 @@ struct StepTiming {
 };
 StepTiming g_timing;
 
-cudaError_t launch_advance_timed(const AdvanceArgs& a, int kperp, int mode, int blocks, size_t smem, cudaStream_t s,
-                                 bool capturing)
+cudaError_t launch_advance_timed(const AdvanceArgs& a, int kperp, int mode, int blocks, int blocks_max, size_t smem,
+                                 cudaStream_t s, bool capturing)
 {
     const int nt = advance_threads(kperp, a.g.dtype, mode, a.g.amr > 0);
     if (!g_timing.on.load(std::memory_order_relaxed) || capturing)
-        return launch_advance(a, g_no_batch, kperp, mode, nt, blocks, smem, s);
+        return launch_advance(a, g_no_batch, kperp, mode, nt, blocks, blocks_max, smem, s);
     std::lock_guard<std::mutex> lock(g_timing.mu);
     const bool rec = g_timing.used + 2 <= (int)g_timing.ev.size();
     if (rec) cudaEventRecord(g_timing.ev[g_timing.used], s);
-    const cudaError_t e = launch_advance(a, g_no_batch, kperp, mode, nt, blocks, smem, s);
+    const cudaError_t e = launch_advance(a, g_no_batch, kperp, mode, nt, blocks, blocks_max, smem, s);
     if (rec) {
         cudaEventRecord(g_timing.ev[g_timing.used + 1], s);
         g_timing.used += 2;
@@ -680,7 +680,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
                 ah[k].n_end = (c0 + chunk < n_end) ? c0 + chunk : n_end;
                 FTE_CUDA(launch_sort(sh[k], hs[k]), "sort launch");
                 FTE_CUDA(cudaMemsetAsync(ah[k].fetch, 0, kFetchBytes, hs[k]), "fetch reset");
-                FTE_CUDA(launch_advance_timed(ah[k], kperp, mode, blocks, smem, hs[k], false), "step kernel launch");
+                FTE_CUDA(launch_advance_timed(ah[k], kperp, mode, blocks, L.blocks, smem, hs[k], false), "step kernel launch");
             }
         }
         FTE_CUDA(cudaEventRecord(side.join, side.s), "join");
@@ -693,7 +693,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
         a.n_end = (c0 + chunk < n_end) ? c0 + chunk : n_end;
         if (sorting) FTE_CUDA(launch_sort(sa, st), "sort launch");
         FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
-        FTE_CUDA(launch_advance_timed(a, kperp, mode, blocks, smem, st, cap != cudaStreamCaptureStatusNone),
+        FTE_CUDA(launch_advance_timed(a, kperp, mode, blocks, L.blocks, smem, st, cap != cudaStreamCaptureStatusNone),
                  "step kernel launch");
         if (nb && mode == kModeSingle)
             FTE_CUDA(launch_reduce(a.part, blocks, (int)nb, t->S, t->S2, t->C, st), "reduce launch");
@@ -1003,7 +1003,7 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
         a.n_end = c1;
         a.n_table0 = c0;
         FTE_CUDA(cudaMemsetAsync(a.fetch, 0, sizeof(unsigned long long), st), "fetch reset");
-        FTE_CUDA(launch_advance(a, g_no_batch, kperp, kModeSingle, kThreads, (int)blocks, smem, st), "step kernel launch");
+        FTE_CUDA(launch_advance(a, g_no_batch, kperp, kModeSingle, kThreads, (int)blocks, (int)max_blocks, smem, st), "step kernel launch");
         if (nb) FTE_CUDA(launch_reduce(a.part, (int)blocks, (int)nb, t->S, t->S2, t->C, st), "reduce launch");
     }
     return FTE_OK;
@@ -1221,7 +1221,7 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
                 ah[k].n_end = (c0 + cfg.steps < n_end) ? c0 + cfg.steps : n_end;
                 FTE_CUDA(launch_sort(sh[k], hs[k]), "sort launch");
                 FTE_CUDA(cudaMemsetAsync(ah[k].fetch, 0, kFetchBytes, hs[k]), "fetch reset");
-                FTE_CUDA(launch_advance(ah[k], bh[k], kperp, cfg.mode, cfg.nt, blocks, smem, hs[k]),
+                FTE_CUDA(launch_advance(ah[k], bh[k], kperp, cfg.mode, cfg.nt, blocks, L.blocks, smem, hs[k]),
                          "step kernel launch");
             }
         }
@@ -1235,7 +1235,7 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
         a.n_end = (c0 + cfg.steps < n_end) ? c0 + cfg.steps : n_end;
         if (sorting) FTE_CUDA(launch_sort(sa, st), "sort launch");
         FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
-        FTE_CUDA(launch_advance(a, b, kperp, cfg.mode, cfg.nt, blocks, smem, st), "step kernel launch");
+        FTE_CUDA(launch_advance(a, b, kperp, cfg.mode, cfg.nt, blocks, L.blocks, smem, st), "step kernel launch");
         if (cfg.mode == kModeShared && nb)
             FTE_CUDA(launch_reduce(a.part, blocks, reduce_bins, t->S, t->S2, t->C, st), "reduce launch");
     }

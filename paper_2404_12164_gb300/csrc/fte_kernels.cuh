@@ -143,9 +143,9 @@ struct AdjK {
 
 // launchers (return cudaGetLastError())
 // step kernel of (kperp, dtype, mode, threads per block); for the single-set modes nt must
-// be advance_threads() of the same arguments
+// be advance_threads() of the same arguments; blocks_max: blocks of one wave
 cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt, int blocks,
-                           size_t smem, cudaStream_t s);
+                           int blocks_max, size_t smem, cudaStream_t s);
 // resident blocks per SM of a step kernel (`pair`: record layout of a single-set kernel)
 cudaError_t advance_occupancy(int kperp, int dtype, int mode, int nt, int pair, int amr, size_t smem,
                               int* blocks_per_sm);
