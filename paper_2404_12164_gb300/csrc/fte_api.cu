@@ -323,6 +323,62 @@ fte_status layout(int device, int kperp, int dtype, int pair, int amr, int mode,
     return FTE_OK;
 }
 
+// Everything fte_inject refuses, for one injection of n particles into P as it stands.
+fte_status inject_check(const fte_particles* P, const fte_background* bg, const fte_inject_spec* spec, uint64_t n,
+                        const fte_tally_buf* t)
+{
+    if (!P || !spec) return fail(FTE_EINVAL, "NULL particles or spec");
+    fte_status s = check_background(bg);
+    if (s != FTE_OK) return s;
+    size_t nb = 0;
+    s = check_tally(t, &nb);
+    if (s != FTE_OK) return s;
+    if (!P->x || !P->y || !P->z || !P->mu || !P->p || !P->w || !P->id || !P->status)
+        return fail(FTE_EINVAL, "NULL particle array");
+    if (P->count + n > P->capacity) return fail(FTE_ENOMEM, "pool capacity %llu < %llu", (unsigned long long)P->capacity,
+                                                (unsigned long long)(P->count + n));
+    if (spec->region != 0 && spec->region != 1) return fail(FTE_EINVAL, "bad region");
+    if (spec->energy != 0 && spec->energy != 1) return fail(FTE_EINVAL, "bad energy mode");
+    if (spec->energy == 0 && !(spec->e0 > 0)) return fail(FTE_EINVAL, "e0 must be > 0");
+    if (spec->energy == 1 && !(spec->e1 > 0 && spec->e2 > spec->e1)) return fail(FTE_EINVAL, "need 0 < e1 < e2");
+    if (spec->region == 1) {
+        if (!(spec->r2 > spec->r1 && spec->r1 > 0)) return fail(FTE_EINVAL, "need 0 < r1 < r2");
+        if (spec->max_tries < 1) return fail(FTE_EINVAL, "max_tries must be >= 1");
+        if (spec->use_divv && (spec->divv_snap < 0 || spec->divv_snap >= resident_snapshots(&bg->grid)))
+            return fail(FTE_EINVAL, "divv_snap out of range");
+    }
+    if (spec->mu_mode == 1 && !(spec->mu0 >= -1.0 && spec->mu0 <= 1.0)) return fail(FTE_EINVAL, "mu0 outside [-1, 1]");
+    if ((uint64_t)spec->id_base + n > 0x100000000ull) return fail(FTE_EINVAL, "particle ids exceed 32 bits");
+    return FTE_OK;
+}
+
+// Kernel-side description of an injection of n particles at pool entry `offset`.
+InjectSet inject_set(const fte_inject_spec* spec, uint64_t offset, uint64_t n)
+{
+    InjectSet a;
+    memset(&a, 0, sizeof(a));
+    a.region = spec->region; a.energy = spec->energy; a.weight = spec->weight; a.mu_mode = spec->mu_mode;
+    a.use_divv = spec->use_divv; a.divv_snap = spec->divv_snap; a.max_tries = spec->max_tries;
+    a.r = (float)spec->r; a.th = (float)spec->th; a.ph = (float)spec->ph;
+    a.r1 = (float)spec->r1; a.r2 = (float)spec->r2; a.th1 = (float)spec->th1; a.th2 = (float)spec->th2;
+    a.ph1 = (float)spec->ph1; a.ph2 = (float)spec->ph2; a.divv_max = (float)spec->divv_max;
+    a.e0 = (float)spec->e0; a.e1 = (float)spec->e1; a.e2 = (float)spec->e2; a.gamma = (float)spec->gamma;
+    a.mu0 = (float)spec->mu0;
+    a.spiral = (float)spec->spiral; a.spiral_rb = (float)spec->spiral_rb;
+    a.seed = spec->seed; a.set_id = spec->set_id; a.id_base = spec->id_base;
+    a.offset = offset; a.n = n;
+    return a;
+}
+
+template <int NS>
+void inject_pool(const fte_particles* P, const fte_background* bg, const fte_tally_buf* t, InjectArgs<NS>* a)
+{
+    a->g = make_gridk(bg);
+    a->x = P->x; a->y = P->y; a->z = P->z; a->mu = P->mu; a->p = P->p; a->w = P->w; a->id = P->id;
+    a->status = P->status;
+    a->ledger_w = t->ledger_w; a->ledger_n = t->ledger_n;
+}
+
 }  // namespace
 
 extern "C" {
@@ -472,28 +528,8 @@ size_t fte_workspace_bytes(int device, const fte_grid* g, const fte_tally_buf* t
 fte_status fte_inject(fte_particles* P, const fte_background* bg, const fte_inject_spec* spec,
                       uint64_t n, const fte_tally_buf* t, uint64_t* n_failed, void* stream)
 {
-    if (!P || !spec) return fail(FTE_EINVAL, "NULL particles or spec");
-    fte_status s = check_background(bg);
+    fte_status s = inject_check(P, bg, spec, n, t);
     if (s != FTE_OK) return s;
-    size_t nb = 0;
-    s = check_tally(t, &nb);
-    if (s != FTE_OK) return s;
-    if (!P->x || !P->y || !P->z || !P->mu || !P->p || !P->w || !P->id || !P->status)
-        return fail(FTE_EINVAL, "NULL particle array");
-    if (P->count + n > P->capacity) return fail(FTE_ENOMEM, "pool capacity %llu < %llu", (unsigned long long)P->capacity,
-                                                (unsigned long long)(P->count + n));
-    if (spec->region != 0 && spec->region != 1) return fail(FTE_EINVAL, "bad region");
-    if (spec->energy != 0 && spec->energy != 1) return fail(FTE_EINVAL, "bad energy mode");
-    if (spec->energy == 0 && !(spec->e0 > 0)) return fail(FTE_EINVAL, "e0 must be > 0");
-    if (spec->energy == 1 && !(spec->e1 > 0 && spec->e2 > spec->e1)) return fail(FTE_EINVAL, "need 0 < e1 < e2");
-    if (spec->region == 1) {
-        if (!(spec->r2 > spec->r1 && spec->r1 > 0)) return fail(FTE_EINVAL, "need 0 < r1 < r2");
-        if (spec->max_tries < 1) return fail(FTE_EINVAL, "max_tries must be >= 1");
-        if (spec->use_divv && (spec->divv_snap < 0 || spec->divv_snap >= resident_snapshots(&bg->grid)))
-            return fail(FTE_EINVAL, "divv_snap out of range");
-    }
-    if (spec->mu_mode == 1 && !(spec->mu0 >= -1.0 && spec->mu0 <= 1.0)) return fail(FTE_EINVAL, "mu0 outside [-1, 1]");
-    if ((uint64_t)spec->id_base + n > 0x100000000ull) return fail(FTE_EINVAL, "particle ids exceed 32 bits");
     if (n == 0) {
         if (n_failed) *n_failed = 0;
         return FTE_OK;
@@ -501,22 +537,11 @@ fte_status fte_inject(fte_particles* P, const fte_background* bg, const fte_inje
     cudaStream_t st = (cudaStream_t)stream;
     unsigned long long before = 0;
     if (n_failed) FTE_CUDA(cudaMemcpyAsync(&before, t->ledger_n + 5, sizeof(before), cudaMemcpyDeviceToHost, st), "ledger read");
-    InjectArgs a;
+    InjectArgs<1> a;
     memset(&a, 0, sizeof(a));
-    a.g = make_gridk(bg);
-    a.n_snap = bg->grid.n_snap;
-    a.region = spec->region; a.energy = spec->energy; a.weight = spec->weight; a.mu_mode = spec->mu_mode;
-    a.use_divv = spec->use_divv; a.divv_snap = spec->divv_snap; a.max_tries = spec->max_tries;
-    a.r = (float)spec->r; a.th = (float)spec->th; a.ph = (float)spec->ph;
-    a.r1 = (float)spec->r1; a.r2 = (float)spec->r2; a.th1 = (float)spec->th1; a.th2 = (float)spec->th2;
-    a.ph1 = (float)spec->ph1; a.ph2 = (float)spec->ph2; a.divv_max = (float)spec->divv_max;
-    a.e0 = (float)spec->e0; a.e1 = (float)spec->e1; a.e2 = (float)spec->e2; a.gamma = (float)spec->gamma;
-    a.mu0 = (float)spec->mu0;
-    a.spiral = (float)spec->spiral; a.spiral_rb = (float)spec->spiral_rb;
-    a.seed = spec->seed; a.set_id = spec->set_id; a.id_base = spec->id_base;
-    a.offset = P->count; a.n = n;
-    a.x = P->x; a.y = P->y; a.z = P->z; a.mu = P->mu; a.p = P->p; a.w = P->w; a.id = P->id; a.status = P->status;
-    a.ledger_w = t->ledger_w; a.ledger_n = t->ledger_n;
+    inject_pool(P, bg, t, &a);
+    a.set[0] = inject_set(spec, P->count, n);
+    a.n_sets = 1;
     FTE_CUDA(launch_inject(a, st), "inject launch");
     P->count += n;
     if (n_failed) {
@@ -1330,11 +1355,27 @@ fte_status fte_inject_batched(fte_particles* P, const fte_background* bg, const 
     if (P->count + total > P->capacity) return fail(FTE_ENOMEM, "pool capacity %llu < %llu",
                                                     (unsigned long long)P->capacity,
                                                     (unsigned long long)(P->count + total));
+    // the sets in order up to the first that is refused, all in one launch: the sets before it
+    // are injected and the call returns its status
+    InjectArgs<FTE_MAX_SETS> a;
+    memset(&a, 0, sizeof(a));
+    fte_status result = FTE_OK;
     for (int s = 0; s < n_sets; ++s) {
-        const fte_status st = fte_inject(P, bg, specs + s, counts[s], t, nullptr, stream);
-        if (st != FTE_OK) return st;
+        result = inject_check(P, bg, specs + s, counts[s], t);
+        if (result != FTE_OK) break;
+        if (counts[s] == 0) continue;
+        a.set[a.n_sets++] = inject_set(specs + s, P->count, counts[s]);
+        P->count += counts[s];
     }
-    return FTE_OK;
+    if (a.n_sets > 0) {
+        inject_pool(P, bg, t, &a);
+        const cudaError_t e = launch_inject(a, (cudaStream_t)stream);
+        if (e != cudaSuccess) {
+            P->count = a.set[0].offset;
+            return cuda_fail(e, "inject launch");
+        }
+    }
+    return result;
 }
 
 fte_status fte_advance_batched(fte_particles* P, const fte_background* bg, const fte_params* prm,

@@ -93,18 +93,27 @@ struct ObsOut {
     double e_lo, e_hi, t_lo, t_hi;
 };
 
-struct InjectArgs {
-    GridK g;
-    int n_snap, region, energy, weight, mu_mode, use_divv, divv_snap, max_tries;
+// One injection (the particles of one parameter set).
+struct InjectSet {
+    int region, energy, weight, mu_mode, use_divv, divv_snap, max_tries;
+    unsigned block0;              // first block of this set's particles
     float r, th, ph, r1, r2, th1, th2, ph1, ph2, divv_max, e0, e1, e2, gamma, mu0;
     float spiral, spiral_rb;      // box: longitude = sampled spiral phase - spiral (r - spiral_rb)
     uint32_t seed, set_id, id_base;
-    unsigned long long offset, n;
+    unsigned long long offset, n; // pool entries [offset, offset + n)
+};
+
+// NS injections in one launch: NS = 1, or up to FTE_MAX_SETS of an ensemble.
+template <int NS>
+struct InjectArgs {
+    GridK g;
+    int n_sets;
     float *x, *y, *z, *mu, *p, *w;
     uint32_t* id;
     uint8_t* status;
     double* ledger_w;
     unsigned long long* ledger_n;
+    InjectSet set[NS];
 };
 
 static_assert(sizeof(AdvanceArgs) + sizeof(BatchArgs) <= 4096, "step kernel parameters exceed 4 KB");
@@ -177,7 +186,9 @@ cudaError_t launch_tally_out(const double* S, const double* S2, const unsigned l
                              const ObsOut& ob, int kind, double* out, cudaStream_t s);
 cudaError_t launch_convolve(const double* S, const ObsOut& ob, int kind, const double* src, double* out,
                             cudaStream_t s);
-cudaError_t launch_inject(const InjectArgs& a, cudaStream_t s);
+// a.set[].block0 are filled in here
+template <int NS>
+cudaError_t launch_inject(InjectArgs<NS>& a, cudaStream_t s);
 // adjoint (fte_adjoint.cu)
 // resident blocks per SM of an adjoint kernel (kind 0 forward, 1 backward VJP, 2 replay)
 cudaError_t adjoint_blocks(int dtype, int pair, int kind, int* blocks_per_sm);

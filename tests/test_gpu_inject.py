@@ -1,0 +1,95 @@
+"""Injection where the warp shares its position attempts: the accepted attempt of every particle
+is the first one that the oracle, trying one after another, accepts.
+
+Sizes where a warp has one particle or is partly empty, attempt limits below, at and beyond what
+one round evaluates, failed injections, and ensembles whose sets end inside a block.  Positions
+agree to FP32 rounding (r, theta and phi each carry a few rounded operations on values of order
+1: 1e-5); particles whose acceptance the oracle marks as within rounding are left out."""
+import dataclasses
+import math
+
+import numpy as np
+import pytest
+
+from fte_inputs import configs
+from oracle import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cir():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from oracle import build as ob
+    from paper_2404_12164_gb300 import api, build
+    build.build()
+    ob.build()
+    w = configs.scaled(configs.cir_uniform_1e6(), nr=64, nth=16, nph=32, n_snap=1)
+    w.grid.periodic = False
+    f = configs.build_background(w)
+    bg = api.Background(w.grid)
+    api.fte_load_background(bg, f)
+    return w, bg, O.grid_background(w.grid, f)
+
+
+def _compare(st, ref):
+    ok = (ref["flags"] & 1) == 0
+    # the oracle alone sets the mark: about 8e-4 per attempt, at most about 20 attempts a particle
+    assert (~ok).sum() <= 1 + 0.05 * len(ok)
+    assert np.array_equal(st["status"][ok], ref["status"][ok])
+    for k in ("x", "y", "z"):
+        assert np.abs(st[k] - ref[k])[ok].max() < 1e-5, k
+    assert np.abs(st["w"] - ref["w"])[ok].max() < 1e-5
+    # E = q^(-1/2) with q = lo + u (hi - lo) between 400 and 0.04 (E^-3 over 50 keV - 5 MeV): q is
+    # rounded at the size of lo, so dE / E <= 2^-23 lo / (2 q) and dp / p about half of dE / E
+    E = 938.27208816 * ref["p"] ** 2 / (np.sqrt(1 + ref["p"] ** 2) + 1)
+    assert (np.abs(st["p"] / ref["p"] - 1) <= 1e-5 + 2.0 ** -23 * 400 * E ** 2 / 2)[ok].all()
+    assert np.array_equal(st["id"], ref["id"])
+
+
+@pytest.mark.parametrize("max_tries", [1, 2, 5, 33, 256])
+@pytest.mark.parametrize("n", [1, 33, 255, 1000])
+def test_first_accepted_attempt(cir, n, max_tries):
+    from paper_2404_12164_gb300 import api
+    w, bg, obg = cir
+    spec = dataclasses.replace(w.inject, max_tries=max_tries, seed=n + max_tries, energy="powerlaw")
+    pool, tally = api.Particles(n), api.Tally([])
+    failed = api.fte_inject(pool, bg, spec, n, tally)
+    ref, _ = O.inject(obg, spec, np.arange(n))
+    st = pool.state()
+    _compare(st, ref)
+    lw, ln = api.fte_ledger(tally)
+    assert failed == ln[5] == (st["status"] == O.INJ_FAIL).sum() and ln[0] == n - failed
+    assert lw[0] == pytest.approx(st["w"].astype(np.float64).sum(), rel=1e-12)
+
+
+@pytest.mark.parametrize("counts", [(1,), (33, 1, 256), (0, 257, 0, 31, 700)])
+def test_sets_in_one_launch(cir, counts):
+    from paper_2404_12164_gb300 import api
+    w, bg, obg = cir
+    sets = [configs.EnsembleSet(0.1 + s, w.params.q, 0.05, 0.048, s, s, c,
+                                dataclasses.replace(w.inject, seed=s, set_id=s, e0=0.02 * (s + 1)))
+            for s, c in enumerate(counts)]
+    pool, tally = api.Particles(sum(counts)), api.Tally([], n_sets=len(counts))
+    api.fte_inject_batched(pool, bg, sets, tally)
+    st = pool.state()
+    a = 0
+    for e in sets:
+        ref, _ = O.inject(obg, e.inject, np.arange(e.count))
+        if e.count:
+            _compare({k: v[a:a + e.count] for k, v in st.items()}, ref)
+        a += e.count
+    assert api.fte_ledger(tally)[1][0] == (st["status"] == 0).sum()
+
+
+def test_refused_set_keeps_the_sets_before_it(cir):
+    from paper_2404_12164_gb300 import api
+    w, bg, _ = cir
+    good = configs.EnsembleSet(0.1, w.params.q, 0.05, 0.048, 0, 0, 40, w.inject)
+    bad = dataclasses.replace(good, inject=dataclasses.replace(w.inject, r1=2.0, r2=1.0))
+    pool, tally = api.Particles(80), api.Tally([], n_sets=2)
+    with pytest.raises(Exception):
+        api.fte_inject_batched(pool, bg, [good, bad], tally)
+    assert pool.count == 40 and api.fte_ledger(tally)[1][0] + api.fte_ledger(tally)[1][5] == 40
