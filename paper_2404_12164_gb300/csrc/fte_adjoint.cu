@@ -20,6 +20,9 @@
 
 namespace fte {
 
+// the form of the forward and replay steps (adjoint passes of 2e5 particles 43.3 -> 42.6 ms)
+constexpr int kAdjShape = kShapeUnroll | kShapeNormals;
+
 // ---------------------------------------------------------------------------
 // d/dq and d/dH (quasi-linear) or d/deps (Eq. 5) of the normalisation integral,
 // same nodes as launch_norm: mu = s^3, Simpson on [0, 1] in s.
@@ -167,7 +170,8 @@ __device__ __forceinline__ void dmumu_vjp(const ParamsK& P, float I, float rq, f
 }
 
 // ---------------------------------------------------------------------------
-// Vector-Jacobian product of one step (lambda_perp = 0): lam holds the adjoint
+// Vector-Jacobian product of one step (lambda_perp = 0); OPT fixes the grid's options only, so
+// that the rest is contracted into the same fused multiply-adds in every build: lam holds the adjoint
 // of the state after step n on entry and of the state before it on return.
 // Score form (win > 0): when the pitch-angle Gaussian's mean m lies within win
 // widths s of a value landing at mu = 0, mu' is held instead of differentiated:
@@ -176,7 +180,7 @@ __device__ __forceinline__ void dmumu_vjp(const ParamsK& P, float I, float rq, f
 // the place of the adjoint of mu'; m and s then carry it back to the state and
 // the parameters exactly as the pathwise adjoint would.
 // ---------------------------------------------------------------------------
-template <int DT, int LAY>
+template <int DT, int LAY, int OPT>
 __device__ void step_vjp(const AdvanceArgs& a, float I, float rq, float rh, long long n, uint32_t pid, float x,
                          float y, float z, float mu, float p, const float* sc, float Gto, float win, float* lam,
                          float* gth)
@@ -196,7 +200,7 @@ __device__ void step_vjp(const AdvanceArgs& a, float I, float rq, float rh, long
     float ph = atan2f(y, x);
     if (ph < 0.f) ph += kTwoPi;
     Loc L;
-    locate(g, r, th, ph, L);
+    locate<OPT>(g, r, th, ph, L);
     Fields<false> F;
     gather<false, DT, LAY>(g, e, L, sc, F);
     const float* B = F.f;
@@ -391,8 +395,8 @@ __device__ void step_vjp(const AdvanceArgs& a, float I, float rq, float rh, long
 // in spatial order from a.order when reordering is on) stores its checkpoint,
 // runs the segment's steps and adds its observable to J_part.
 // ---------------------------------------------------------------------------
-template <int DT, int LAY>
-__global__ void __launch_bounds__(256) adj_forward_kernel(const AdvanceArgs a, const AdjK k)
+template <int DT, int LAY, int OPT>
+__global__ void __launch_bounds__(256, 2) adj_forward_kernel(const AdvanceArgs a, const AdjK k)
 {
     __shared__ float sc[FTE_NFIELD];
     __shared__ double red[8];
@@ -420,11 +424,11 @@ __global__ void __launch_bounds__(256) adj_forward_kernel(const AdvanceArgs a, c
         double J = 0.0;
         int st = FTE_ALIVE;
         long long s = a.n_start;
+        float r = radius(x, y, z);
         for (; s < a.n_end; ++s) {
-            const float r = sqrtf(x * x + y * y + z * z);
             J += (double)(w * a.prm.dt * smooth_k(k, r, p, time_arg(k, s), nullptr, nullptr));
-            st = step<false, DT, kModeSingle, LAY>(a, a.prm, I, 0, s, pid, x, y, z, mu, p, w, nullptr, nullptr,
-                                              nullptr, sc, noor, nrun);
+            st = step<false, DT, kModeNoTally, LAY, OPT, kAdjShape>(a, a.prm, I, 0, s, pid, x, y, z, mu, p, r, w,
+                                                                    nullptr, nullptr, nullptr, sc, noor, nrun);
             if (st != FTE_ALIVE) { ++s; break; }
         }
         // steps taken since the start of the run (a.n_table0), counting the one that ended it
@@ -455,8 +459,8 @@ __global__ void __launch_bounds__(256) adj_forward_kernel(const AdvanceArgs a, c
 // the stored states, carrying the adjoints between launches in k.adj.  The launch
 // of the run's first chunk adds the injection-index term and reduces the gradients.
 // ---------------------------------------------------------------------------
-template <int DT, int LAY>
-__global__ void __launch_bounds__(256) adj_replay_kernel(const AdvanceArgs a, const AdjK k)
+template <int DT, int LAY, int OPT>
+__global__ void __launch_bounds__(256, 2) adj_replay_kernel(const AdvanceArgs a, const AdjK k)
 {
     __shared__ float sc[FTE_NFIELD];
     if (DT != FTE_F32 && threadIdx.x < FTE_NFIELD) sc[threadIdx.x] = __ldg(a.g.scale + threadIdx.x);
@@ -484,12 +488,13 @@ __global__ void __launch_bounds__(256) adj_replay_kernel(const AdvanceArgs a, co
         const float w = a.w[i];
         const uint32_t pid = a.id[i];
         const long long hi = min(ce, e);
+        float r = radius(x, y, z);
         for (long long s = cs; s < hi; ++s) {
             float* sp = k.scratch + (size_t)(s - n0) * 5 * n + f;
             sp[0] = x; sp[n] = y; sp[2 * n] = z; sp[3 * n] = mu; sp[4 * n] = p;
             if (s + 1 < e)
-                step<false, DT, kModeSingle, LAY>(a, a.prm, I, 0, s, pid, x, y, z, mu, p, w, nullptr, nullptr, nullptr,
-                                             sc, noor, nrun);
+                step<false, DT, kModeNoTally, LAY, OPT, kAdjShape>(a, a.prm, I, 0, s, pid, x, y, z, mu, p, r, w,
+                                                                   nullptr, nullptr, nullptr, sc, noor, nrun);
         }
         if (ce < e) {      // the start of the next chunk
             float* cp = k.carry + i;
@@ -498,7 +503,7 @@ __global__ void __launch_bounds__(256) adj_replay_kernel(const AdvanceArgs a, co
     }
 }
 
-template <int DT, int LAY>
+template <int DT, int LAY, int OPT>
 __global__ void __launch_bounds__(256, 2) adj_back_kernel(const AdvanceArgs a, const AdjK k)
 {
     __shared__ float sc[FTE_NFIELD];
@@ -538,7 +543,7 @@ __global__ void __launch_bounds__(256, 2) adj_back_kernel(const AdvanceArgs a, c
         for (long long s = min(ce, e) - 1; s >= cs; --s) {
             const float* sp = k.scratch + (size_t)(s - n0) * 5 * n + f;
             const float sx = sp[0], sy = sp[n], sz = sp[2 * n], smu = sp[3 * n], spp = sp[4 * n];
-            step_vjp<DT, LAY>(a, I, rq, rh, s, pid, sx, sy, sz, smu, spp, sc, Gacc, k.lr_window, lam, gth);
+            step_vjp<DT, LAY, OPT>(a, I, rq, rh, s, pid, sx, sy, sz, smu, spp, sc, Gacc, k.lr_window, lam, gth);
             // the observable's own term at the start-of-step state
             const float r = sqrtf(sx * sx + sy * sy + sz * sz);
             float dKdr, dKdp;
@@ -584,48 +589,43 @@ __global__ void __launch_bounds__(256, 2) adj_back_kernel(const AdvanceArgs a, c
     }
 }
 
-template <int LAY>
-static const void* fwd_fn_lay(int dtype)
+// one adjoint kernel: kind 0 forward, 1 backward VJP, 2 replay
+template <int DT, int LAY, int OPT>
+static const void* adj_kernel(int kind)
 {
-    if (dtype == FTE_BF16) return (const void*)adj_forward_kernel<FTE_BF16, LAY>;
-    if (dtype == FTE_F16) return (const void*)adj_forward_kernel<FTE_F16, LAY>;
-    return (const void*)adj_forward_kernel<FTE_F32, LAY>;
+    if (kind == 1) return (const void*)adj_back_kernel<DT, LAY, OPT>;
+    if (kind == 2) return (const void*)adj_replay_kernel<DT, LAY, OPT>;
+    return (const void*)adj_forward_kernel<DT, LAY, OPT>;
 }
 
-template <int LAY>
-static const void* rep_fn_lay(int dtype)
+template <int LAY, int OPT>
+static const void* adj_fn_dtype(int kind, int dtype)
 {
-    if (dtype == FTE_BF16) return (const void*)adj_replay_kernel<FTE_BF16, LAY>;
-    if (dtype == FTE_F16) return (const void*)adj_replay_kernel<FTE_F16, LAY>;
-    return (const void*)adj_replay_kernel<FTE_F32, LAY>;
+    if (dtype == FTE_BF16) return adj_kernel<FTE_BF16, LAY, OPT>(kind);
+    if (dtype == FTE_F16) return adj_kernel<FTE_F16, LAY, OPT>(kind);
+    return adj_kernel<FTE_F32, LAY, OPT>(kind);
 }
 
-template <int LAY>
-static const void* back_fn_lay(int dtype)
-{
-    if (dtype == FTE_BF16) return (const void*)adj_back_kernel<FTE_BF16, LAY>;
-    if (dtype == FTE_F16) return (const void*)adj_back_kernel<FTE_F16, LAY>;
-    return (const void*)adj_back_kernel<FTE_F32, LAY>;
-}
+int adjoint_opt(const GridK& g, const ParamsK& prm) { return advance_opt(g, prm, 0, kModeSingleGlobal); }
 
-// record layout fixed at compile time, as for the step kernels; kind 0 forward,
-// 1 backward VJP, 2 replay
-static const void* adj_fn(int kind, int dtype, int pair)
+// record layout and, for the common options (advance_opt: cell records only), the options fixed
+// at compile time, as for the step kernels
+static const void* adj_fn(int kind, int dtype, int pair, int opt)
 {
-    if (kind == 1) return pair ? back_fn_lay<kLayPair>(dtype) : back_fn_lay<kLayCell>(dtype);
-    if (kind == 2) return pair ? rep_fn_lay<kLayPair>(dtype) : rep_fn_lay<kLayCell>(dtype);
-    return pair ? fwd_fn_lay<kLayPair>(dtype) : fwd_fn_lay<kLayCell>(dtype);
+    if (opt == kOptLinear) return adj_fn_dtype<kLayCell, kOptLinear>(kind, dtype);
+    if (opt == kOptAmrLog) return adj_fn_dtype<kLayCell, kOptAmrLog>(kind, dtype);
+    return pair ? adj_fn_dtype<kLayPair, kOptAny>(kind, dtype) : adj_fn_dtype<kLayCell, kOptAny>(kind, dtype);
 }
 
 cudaError_t adjoint_blocks(int dtype, int pair, int kind, int* blocks_per_sm)
 {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, adj_fn(kind, dtype, pair), 256, 0);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, adj_fn(kind, dtype, pair, kOptAny), 256, 0);
 }
 
 static cudaError_t launch_adj(int kind, const AdvanceArgs& a, const AdjK& k, int blocks, cudaStream_t s)
 {
     void* args[] = {(void*)&a, (void*)&k};
-    return cudaLaunchKernel(adj_fn(kind, a.g.dtype, a.g.pair), dim3(blocks), dim3(256), args, 0, s);
+    return cudaLaunchKernel(adj_fn(kind, a.g.dtype, a.g.pair, adjoint_opt(a.g, a.prm)), dim3(blocks), dim3(256), args, 0, s);
 }
 
 cudaError_t launch_adjoint_forward(const AdvanceArgs& a, const AdjK& k, int blocks, cudaStream_t s)

@@ -5,36 +5,76 @@
 
 namespace fte {
 
+// single-set kernels without cross-field diffusion are compiled for exactly the two blocks of
+// 256 threads per SM that they get: told so, the compiler uses all 128 registers and keeps more
+// record loads in flight (left to itself it took 104 - 110; 1e6 particles over 4 days of
+// snapshots 603 -> 577 ms, 1e4 Parker particles 14.8 -> 13.2 ms).  The cross-field builds use
+// 128 anyway and measured 2 % faster left alone.
+constexpr int kMinBlocks = 512 / kThreads;
+
+template <int DT, int MODE, int LAY, int SHAPE>
+static const void* single_dt(int kperp)
+{
+    return kperp ? (const void*)advance_kernel<true, DT, MODE, kThreads, LAY>
+                 : (const void*)advance_kernel<false, DT, MODE, kThreads, LAY, kMinBlocks, kOptAny, SHAPE>;
+}
+
 template <int MODE, int LAY>
 static const void* single_fn(int kperp, int dtype)
 {
-    if (dtype == FTE_BF16)
-        return kperp ? (const void*)advance_kernel<true, FTE_BF16, MODE, kThreads, LAY>
-                     : (const void*)advance_kernel<false, FTE_BF16, MODE, kThreads, LAY>;
-    if (dtype == FTE_F16)
-        return kperp ? (const void*)advance_kernel<true, FTE_F16, MODE, kThreads, LAY>
-                     : (const void*)advance_kernel<false, FTE_F16, MODE, kThreads, LAY>;
-    return kperp ? (const void*)advance_kernel<true, FTE_F32, MODE, kThreads, LAY>
-                 : (const void*)advance_kernel<false, FTE_F32, MODE, kThreads, LAY>;
+    constexpr int shape = MODE == kModeSingle ? kShapeNormals : kShapeLoop;
+    if (dtype == FTE_BF16) return single_dt<FTE_BF16, MODE, LAY, shape>(kperp);
+    if (dtype == FTE_F16) return single_dt<FTE_F16, MODE, LAY, shape>(kperp);
+    return single_dt<FTE_F32, MODE, LAY, shape>(kperp);
 }
 
-// the register-limited builds of block AMR (global tally, no cross-field diffusion):
-// 16-bit records 3 blocks of 256 threads per SM (at most 85 registers), FP32 records
-// 5 blocks of 128 (at most 102)
+// the builds of block AMR (global tally, no cross-field diffusion): 16-bit records 3 blocks of
+// 256 threads per SM (at most 85 registers), FP32 records 4 blocks of 128 (128 registers, 16
+// warps).  With the options fixed and the shorter step the 16-warp build overtook the 20 warps
+// at 102 registers that FP32 ran before (1e7 particles x 320 steps: 145 ms with 20 warps and 160
+// bytes of spills, 136 with 16; 12 warps at 168 registers 157; 153 before).
 constexpr int kDenseBlocks = 768 / kThreads;
 constexpr int kAmr32Threads = 128;
-constexpr int kAmr32Blocks = 5;
-template <int LAY>
+constexpr int kAmr32Blocks = 4;
+template <int LAY, int OPT = kOptAny, int SHAPE = kShapeLoop>
 static const void* dense_fn(int dtype)
 {
-    if (dtype == FTE_BF16) return (const void*)advance_kernel<false, FTE_BF16, kModeSingleGlobal, kThreads, LAY, kDenseBlocks>;
-    if (dtype == FTE_F16) return (const void*)advance_kernel<false, FTE_F16, kModeSingleGlobal, kThreads, LAY, kDenseBlocks>;
-    return (const void*)advance_kernel<false, FTE_F32, kModeSingleGlobal, kAmr32Threads, LAY, kAmr32Blocks>;
+    if (dtype == FTE_BF16)
+        return (const void*)advance_kernel<false, FTE_BF16, kModeSingleGlobal, kThreads, LAY, kDenseBlocks, OPT, SHAPE>;
+    if (dtype == FTE_F16)
+        return (const void*)advance_kernel<false, FTE_F16, kModeSingleGlobal, kThreads, LAY, kDenseBlocks, OPT, SHAPE>;
+    return (const void*)advance_kernel<false, FTE_F32, kModeSingleGlobal, kAmr32Threads, LAY, kAmr32Blocks, OPT, SHAPE>;
+}
+
+// near: the build with the reach test of the observers (kShapeNear)
+template <int DT>
+static const void* linear_dt(bool near)
+{
+    constexpr int shape = kShapeUnroll | kShapeNormals;
+    return near ? (const void*)advance_kernel<false, DT, kModeSingleGlobal, kThreads, kLayCell, kMinBlocks, kOptLinear,
+                                              shape | kShapeNear>
+                : (const void*)advance_kernel<false, DT, kModeSingleGlobal, kThreads, kLayCell, kMinBlocks, kOptLinear,
+                                              shape>;
+}
+
+static const void* linear_fn(int dtype, bool near)
+{
+    if (dtype == FTE_BF16) return linear_dt<FTE_BF16>(near);
+    if (dtype == FTE_F16) return linear_dt<FTE_F16>(near);
+    return linear_dt<FTE_F32>(near);
 }
 
 static bool dense_variant(int kperp, int mode, int amr)
 {
     return mode == kModeSingleGlobal && !kperp && amr;
+}
+
+int advance_opt(const GridK& g, const ParamsK& prm, int kperp, int mode)
+{
+    const bool common = prm.dmumu == 0 && !prm.use_rig && prm.p_update == 0 && prm.dvdt_term;
+    if (!common || kperp || g.pair || !global_tally(mode)) return kOptAny;
+    if (g.amr > 0) return g.radial && mode == kModeSingleGlobal ? kOptAmrLog : kOptAny;
+    return g.radial ? kOptAny : kOptLinear;
 }
 
 int advance_threads(int kperp, int dtype, int mode, int amr)
@@ -43,11 +83,14 @@ int advance_threads(int kperp, int dtype, int mode, int amr)
 }
 
 // the single-set kernels come in one variant per record layout (pair: 1) and tally
-// mode, and for block AMR in a register-limited build
-static const void* advance_fn(int kperp, int dtype, int mode, int nt, int pair, int amr)
+// mode, for block AMR in a register-limited build, and for the common options (advance_opt)
+// in one with these fixed
+static const void* advance_fn(int kperp, int dtype, int mode, int nt, int pair, int amr, int opt, bool near = true)
 {
-    if (!single_set(mode)) return advance_fn_batched(kperp, dtype, mode, nt, pair);
+    if (!single_set(mode)) return advance_fn_batched(kperp, dtype, mode, nt, pair, opt);
     if (nt != advance_threads(kperp, dtype, mode, amr)) return nullptr;
+    if (opt == kOptAmrLog) return dense_fn<kLayCell, kOptAmrLog, kShapeNear>(dtype);
+    if (opt == kOptLinear) return linear_fn(dtype, near);
     if (dense_variant(kperp, mode, amr)) return pair ? dense_fn<kLayPair>(dtype) : dense_fn<kLayCell>(dtype);
     if (mode == kModeSingleGlobal)
         return pair ? single_fn<kModeSingleGlobal, kLayPair>(kperp, dtype)
@@ -55,10 +98,10 @@ static const void* advance_fn(int kperp, int dtype, int mode, int nt, int pair, 
     return pair ? single_fn<kModeSingle, kLayPair>(kperp, dtype) : single_fn<kModeSingle, kLayCell>(kperp, dtype);
 }
 
-cudaError_t advance_occupancy(int kperp, int dtype, int mode, int nt, int pair, int amr, size_t smem,
+cudaError_t advance_occupancy(int kperp, int dtype, int mode, int nt, int pair, int amr, int opt, size_t smem,
                               int* blocks_per_sm)
 {
-    const void* fn = advance_fn(kperp, dtype, mode, nt, pair, amr);
+    const void* fn = advance_fn(kperp, dtype, mode, nt, pair, amr, opt);
     if (!fn) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -66,21 +109,25 @@ cudaError_t advance_occupancy(int kperp, int dtype, int mode, int nt, int pair, 
 }
 
 cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt, int blocks,
-                           int blocks_max, size_t smem, cudaStream_t s)
+                           size_t smem, cudaStream_t s)
 {
     if (!single_set(mode)) return launch_advance_batched(a, b, kperp, mode, nt, blocks, smem, s);
-    const void* fn = advance_fn(kperp, a.g.dtype, mode, nt, a.g.pair, a.g.amr > 0);
+    // reordered, or at most one particle per thread (see kShapeNear)
+    const bool near = a.order || a.n_particles <= (unsigned long long)blocks * nt;
+    const void* fn = advance_fn(kperp, a.g.dtype, mode, nt, a.g.pair, a.g.amr > 0, advance_opt(a.g, a.prm, kperp, mode),
+                                near);
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {(void*)&a, (void*)&b};
-    // A pool that is not reordered and leaves threads of one wave idle is launched in blocks of
-    // one warp: 1e4 particles in blocks of 256 occupy 40 of 152 SMs with 8 warps each, in blocks
-    // of 32 every SM with 2, and a step's latency falls with the warps it shares an SM with
-    // (1e4 particles x 8640 steps 19.1 -> 17.4 ms, 2000 x 200 0.54 -> 0.50 ms).  From one wave on
-    // the blocks fill every SM anyway.  Global tally only: a block of the shared-memory tally
-    // carries a whole histogram.
-    if (mode == kModeSingleGlobal && !a.order && a.n_particles < (unsigned long long)blocks_max * nt) {
+    // A pool that is not reordered is launched in blocks of one warp, which spread evenly over the
+    // SMs: 1e4 particles in blocks of 256 occupy 40 of 152 SMs with 8 warps each, in blocks of 32
+    // every SM with 2, and a step's latency falls with the warps it shares an SM with (1e4
+    // particles x 8640 steps 19.1 -> 17.4 ms, 2000 x 200 0.54 -> 0.50 ms); 1.3e5 particles, two
+    // per thread, are 248 blocks of 256, two on 96 SMs and one on 56.  Global tally only: a block
+    // of the shared-memory tally carries a whole histogram.
+    if (mode == kModeSingleGlobal && !a.order) {
+        const unsigned long long warps = (a.n_particles + 31) / 32, given = (unsigned long long)blocks * (nt / 32);
+        blocks = (int)(warps < given ? warps : given);
         nt = 32;
-        blocks = (int)((a.n_particles + 31) / 32);
     }
     return cudaLaunchKernel(fn, dim3(blocks), dim3(nt), args, smem, s);
 }

@@ -196,9 +196,12 @@ const BatchArgs g_no_batch = {};    // the single-set kernels ignore their ensem
 void fill_observers(const fte_tally_buf* t, AdvanceArgs* a)
 {
     size_t off = 0;
+    a->any_slab = 0;
+    for (int o = t->n_obs; o < FTE_MAX_OBS; ++o) a->obs[o].dr = -1.f;    // never reached
     for (int o = 0; o < t->n_obs; ++o) {
         const fte_observer& ob = t->obs[o];
         ObsK& k = a->obs[o];
+        if (ob.kind == 2) a->any_slab = 1;
         k.kind = ob.kind; k.ne = ob.ne; k.nt = ob.nt; k.off = (int)off;
         k.r = (float)ob.r; k.dr = (float)ob.dr; k.th = (float)ob.th; k.dth = (float)ob.dth;
         k.ph = (float)ob.ph; k.dph = (float)ob.dph;
@@ -265,16 +268,16 @@ struct StepTiming {
 };
 StepTiming g_timing;
 
-cudaError_t launch_advance_timed(const AdvanceArgs& a, int kperp, int mode, int blocks, int blocks_max, size_t smem,
-                                 cudaStream_t s, bool capturing)
+cudaError_t launch_advance_timed(const AdvanceArgs& a, int kperp, int mode, int blocks, size_t smem, cudaStream_t s,
+                                 bool capturing)
 {
     const int nt = advance_threads(kperp, a.g.dtype, mode, a.g.amr > 0);
     if (!g_timing.on.load(std::memory_order_relaxed) || capturing)
-        return launch_advance(a, g_no_batch, kperp, mode, nt, blocks, blocks_max, smem, s);
+        return launch_advance(a, g_no_batch, kperp, mode, nt, blocks, smem, s);
     std::lock_guard<std::mutex> lock(g_timing.mu);
     const bool rec = g_timing.used + 2 <= (int)g_timing.ev.size();
     if (rec) cudaEventRecord(g_timing.ev[g_timing.used], s);
-    const cudaError_t e = launch_advance(a, g_no_batch, kperp, mode, nt, blocks, blocks_max, smem, s);
+    const cudaError_t e = launch_advance(a, g_no_batch, kperp, mode, nt, blocks, smem, s);
     if (rec) {
         cudaEventRecord(g_timing.ev[g_timing.used + 1], s);
         g_timing.used += 2;
@@ -293,8 +296,19 @@ struct SideStream {
     }
 };
 
-fte_status layout(int device, int kperp, int dtype, int pair, int amr, int mode, size_t nbins, long long n_steps,
-                  size_t sort_bytes, WsLayout* L)
+// The compile-time options of the step kernel for these parameters (advance_opt).  The
+// workspace of the global-tally kernels does not depend on them.
+int params_opt(const GridK& g, const fte_params* prm, int kperp, int mode)
+{
+    ParamsK k;
+    memset(&k, 0, sizeof(k));
+    k.dmumu = prm->dmumu; k.p_update = prm->p_update; k.dvdt_term = prm->dvdt_term;
+    k.use_rig = (prm->p_ref > 0.0 && prm->alpha != 0.0) ? 1 : 0;
+    return advance_opt(g, k, kperp, mode);
+}
+
+fte_status layout(int device, int kperp, int dtype, int pair, int amr, int mode, int opt, size_t nbins,
+                  long long n_steps, size_t sort_bytes, WsLayout* L)
 {
     const int sms = device_sms(device);
     if (sms <= 0) return fail(FTE_ECUDA, "cannot query device %d", device);
@@ -304,7 +318,7 @@ fte_status layout(int device, int kperp, int dtype, int pair, int amr, int mode,
     FTE_CUDA(cudaGetDevice(&cur), "cudaGetDevice");
     if (cur != device) FTE_CUDA(cudaSetDevice(device), "cudaSetDevice");
     L->threads = advance_threads(kperp, dtype, mode, amr);
-    cudaError_t e = advance_occupancy(kperp, dtype, mode, L->threads, pair, amr, smem, &per_sm);
+    cudaError_t e = advance_occupancy(kperp, dtype, mode, L->threads, pair, amr, opt, smem, &per_sm);
     if (cur != device) cudaSetDevice(cur);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
     if (per_sm < 1) return fail(FTE_ENOTSUP, "step kernel does not fit on an SM with %zu bytes of tally", smem);
@@ -518,7 +532,8 @@ size_t fte_workspace_bytes(int device, const fte_grid* g, const fte_tally_buf* t
                 for (int mode : {kModeSingle, kModeSingleGlobal}) {
                     if (mode == kModeSingle && nb > (size_t)kMaxSmemBins) continue;
                     WsLayout L;
-                    if (layout(device, kperp, dtype, pair, g->amr_levels > 0, mode, nb, n_steps, sort_bytes, &L) != FTE_OK)
+                    if (layout(device, kperp, dtype, pair, g->amr_levels > 0, mode, kOptAny, nb, n_steps, sort_bytes,
+                               &L) != FTE_OK)
                         return 0;
                     if (L.total > best) best = L.total;
                 }
@@ -590,7 +605,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
     const GridK gk = make_gridk(bg);
     const int sorting = prm->sort_every > 0;
     WsLayout L;
-    s = layout(device, kperp, bg->grid.dtype, gk.pair, gk.amr > 0, mode, nb, nsteps,
+    s = layout(device, kperp, bg->grid.dtype, gk.pair, gk.amr > 0, mode, params_opt(gk, prm, kperp, mode), nb, nsteps,
                sorting ? advance_sort_bytes(gk, P->count) : 0,
                &L);
     if (s != FTE_OK) return s;
@@ -661,7 +676,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
     const size_t smem = single_smem(mode, nb);
     int per_sm = 0;
     FTE_CUDA(advance_occupancy(kperp, bg->grid.dtype, mode, L.threads, bg->grid.layout == FTE_LAYOUT_PAIR, gk.amr > 0,
-                               smem, &per_sm), "occupancy");
+                               params_opt(gk, prm, kperp, mode), smem, &per_sm), "occupancy");
 
     // Two halves on two streams: while the last particles of one half's launch run, the
     // other half's reordering and launch fill the idle SMs (the step kernel launches one
@@ -705,7 +720,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
                 ah[k].n_end = (c0 + chunk < n_end) ? c0 + chunk : n_end;
                 FTE_CUDA(launch_sort(sh[k], hs[k]), "sort launch");
                 FTE_CUDA(cudaMemsetAsync(ah[k].fetch, 0, kFetchBytes, hs[k]), "fetch reset");
-                FTE_CUDA(launch_advance_timed(ah[k], kperp, mode, blocks, L.blocks, smem, hs[k], false), "step kernel launch");
+                FTE_CUDA(launch_advance_timed(ah[k], kperp, mode, blocks, smem, hs[k], false), "step kernel launch");
             }
         }
         FTE_CUDA(cudaEventRecord(side.join, side.s), "join");
@@ -718,7 +733,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
         a.n_end = (c0 + chunk < n_end) ? c0 + chunk : n_end;
         if (sorting) FTE_CUDA(launch_sort(sa, st), "sort launch");
         FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
-        FTE_CUDA(launch_advance_timed(a, kperp, mode, blocks, L.blocks, smem, st, cap != cudaStreamCaptureStatusNone),
+        FTE_CUDA(launch_advance_timed(a, kperp, mode, blocks, smem, st, cap != cudaStreamCaptureStatusNone),
                  "step kernel launch");
         if (nb && mode == kModeSingle)
             FTE_CUDA(launch_reduce(a.part, blocks, (int)nb, t->S, t->S2, t->C, st), "reduce launch");
@@ -971,7 +986,7 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
     const size_t smem = part_block;
     int per_sm = 0;
     FTE_CUDA(advance_occupancy(kperp, bg->grid.dtype, kModeSingle, kThreads, bg->grid.layout == FTE_LAYOUT_PAIR,
-                                bg->grid.amr_levels > 0, smem, &per_sm), "occupancy");
+                                bg->grid.amr_levels > 0, kOptAny, smem, &per_sm), "occupancy");
     if (per_sm < 1) return fail(FTE_ENOTSUP, "step kernel does not fit on an SM with %zu bytes of tally", smem);
     long long max_blocks = (long long)sms * per_sm;
     if ((size_t)max_blocks > fit) max_blocks = (long long)fit;
@@ -1028,7 +1043,7 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
         a.n_end = c1;
         a.n_table0 = c0;
         FTE_CUDA(cudaMemsetAsync(a.fetch, 0, sizeof(unsigned long long), st), "fetch reset");
-        FTE_CUDA(launch_advance(a, g_no_batch, kperp, kModeSingle, kThreads, (int)blocks, (int)max_blocks, smem, st), "step kernel launch");
+        FTE_CUDA(launch_advance(a, g_no_batch, kperp, kModeSingle, kThreads, (int)blocks, smem, st), "step kernel launch");
         if (nb) FTE_CUDA(launch_reduce(a.part, (int)blocks, (int)nb, t->S, t->S2, t->C, st), "reduce launch");
     }
     return FTE_OK;
@@ -1054,7 +1069,7 @@ size_t ens_smem(int mode, int n_sets, size_t nb)
     return mode == kModeShared ? 3 * sizeof(float) * shared_bins(n_sets, nb) : 0;
 }
 
-fte_status ens_layout(int device, int kperp, int dtype, int pair, int mode, int nt, int n_sets, size_t nb,
+fte_status ens_layout(int device, int kperp, int dtype, int pair, int mode, int opt, int nt, int n_sets, size_t nb,
                       long long n_steps, size_t sort_bytes, EnsLayout* L)
 {
     const int sms = device_sms(device);
@@ -1063,7 +1078,7 @@ fte_status ens_layout(int device, int kperp, int dtype, int pair, int mode, int 
     int per_sm = 0, cur = 0;
     FTE_CUDA(cudaGetDevice(&cur), "cudaGetDevice");
     if (cur != device) FTE_CUDA(cudaSetDevice(device), "cudaSetDevice");
-    cudaError_t e = advance_occupancy(kperp, dtype, mode, nt, pair, 0, smem, &per_sm);
+    cudaError_t e = advance_occupancy(kperp, dtype, mode, nt, pair, 0, opt, smem, &per_sm);
     if (cur != device) cudaSetDevice(cur);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
     if (per_sm < 1) return fail(FTE_ENOTSUP, "ensemble step kernel does not fit on an SM with %zu bytes of tally", smem);
@@ -1127,7 +1142,8 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
     const GridK gk = make_gridk(bg);
     const int sorting = prm->sort_every > 0;
     EnsLayout L;
-    fte_status s = ens_layout(device, kperp, bg->grid.dtype, gk.pair, cfg.mode, cfg.nt, n_sets, nb, nsteps,
+    fte_status s = ens_layout(device, kperp, bg->grid.dtype, gk.pair, cfg.mode, params_opt(gk, prm, kperp, cfg.mode),
+                              cfg.nt, n_sets, nb, nsteps,
                               sorting ? advance_sort_bytes(gk, P->count) : 0, &L);
     if (s != FTE_OK) return s;
     if (ws_bytes < L.total) return fail(FTE_ENOMEM, "workspace has %zu bytes, needs %zu", ws_bytes, L.total);
@@ -1246,7 +1262,7 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
                 ah[k].n_end = (c0 + cfg.steps < n_end) ? c0 + cfg.steps : n_end;
                 FTE_CUDA(launch_sort(sh[k], hs[k]), "sort launch");
                 FTE_CUDA(cudaMemsetAsync(ah[k].fetch, 0, kFetchBytes, hs[k]), "fetch reset");
-                FTE_CUDA(launch_advance(ah[k], bh[k], kperp, cfg.mode, cfg.nt, blocks, L.blocks, smem, hs[k]),
+                FTE_CUDA(launch_advance(ah[k], bh[k], kperp, cfg.mode, cfg.nt, blocks, smem, hs[k]),
                          "step kernel launch");
             }
         }
@@ -1260,7 +1276,7 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
         a.n_end = (c0 + cfg.steps < n_end) ? c0 + cfg.steps : n_end;
         if (sorting) FTE_CUDA(launch_sort(sa, st), "sort launch");
         FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
-        FTE_CUDA(launch_advance(a, b, kperp, cfg.mode, cfg.nt, blocks, L.blocks, smem, st), "step kernel launch");
+        FTE_CUDA(launch_advance(a, b, kperp, cfg.mode, cfg.nt, blocks, smem, st), "step kernel launch");
         if (cfg.mode == kModeShared && nb)
             FTE_CUDA(launch_reduce(a.part, blocks, reduce_bins, t->S, t->S2, t->C, st), "reduce launch");
     }
@@ -1335,7 +1351,7 @@ size_t fte_workspace_bytes_batched(int device, const fte_grid* g, const fte_tall
                     if (mode == kModeShared && !shared_fits(n_sets, nb)) continue;
                     EnsLayout L;
                     for (int pair = 0; pair < 2; ++pair) {
-                        const fte_status s = ens_layout(device, kperp, dtype, pair, mode, nt, n_sets, nb, n_steps,
+                        const fte_status s = ens_layout(device, kperp, dtype, pair, mode, kOptAny, nt, n_sets, nb, n_steps,
                                                         sort_bytes, &L);
                         if (s == FTE_ENOTSUP) continue;
                         if (s != FTE_OK) return 0;
@@ -1636,6 +1652,7 @@ fte_status adj_args(const fte_particles* P, const fte_background* bg, const fte_
         if (nsteps > 0) FTE_CUDA(launch_step_table(ta, st), "step table launch");
     }
     memset(a, 0, sizeof(*a));
+    a->obs[0].dr = -1.f;               // no observers
     a->g = make_gridk(bg);
     a->prm.dmumu = prm->dmumu; a->prm.p_update = prm->p_update; a->prm.kappa_drift = prm->kappa_drift;
     a->prm.dvdt_term = prm->dvdt_term;

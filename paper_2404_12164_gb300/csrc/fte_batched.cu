@@ -26,8 +26,25 @@ static const void* pick_layout(int kperp, int dtype, int pair)
     return pair ? pick<MODE, NT, kLayPair>(kperp, dtype) : pick<MODE, NT, kLayCell>(kperp, dtype);
 }
 
-const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair)
+// global tally, cell records, no cross-field diffusion, options fixed (advance_opt)
+template <int DT, int NT>
+static const void* pick_linear_dt()
 {
+    return (const void*)advance_kernel<false, DT, kModeGlobal, NT, kLayCell, 0, kOptLinear,
+                                       kShapeUnroll | kShapeNormals | kShapeNear>;
+}
+
+template <int NT>
+static const void* pick_linear(int dtype)
+{
+    if (dtype == FTE_BF16) return pick_linear_dt<FTE_BF16, NT>();
+    if (dtype == FTE_F16) return pick_linear_dt<FTE_F16, NT>();
+    return pick_linear_dt<FTE_F32, NT>();
+}
+
+const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair, int opt)
+{
+    if (opt == kOptLinear) return nt == 128 ? pick_linear<128>(dtype) : (nt == 256 ? pick_linear<256>(dtype) : nullptr);
     if (mode == kModeShared) {
         if (nt == 128) return pick_layout<kModeShared, 128>(kperp, dtype, pair);
         if (nt == 256) return pick_layout<kModeShared, 256>(kperp, dtype, pair);
@@ -41,7 +58,7 @@ const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair)
 cudaError_t launch_advance_batched(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt,
                                    int blocks, size_t smem, cudaStream_t s)
 {
-    const void* fn = advance_fn_batched(kperp, a.g.dtype, mode, nt, a.g.pair);
+    const void* fn = advance_fn_batched(kperp, a.g.dtype, mode, nt, a.g.pair, advance_opt(a.g, a.prm, kperp, mode));
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {(void*)&a, (void*)&b};
     return cudaLaunchKernel(fn, dim3(blocks), dim3(nt), args, smem, s);

@@ -119,17 +119,35 @@ __device__ __forceinline__ float energy_of(float p)
 }
 
 // ---------------------------------------------------------------------------
+// Options fixed at compile time.  The step's options are the same for every particle of a
+// launch, but each costs a parameter load, a test and a branch per step, and the branches cut
+// the step into short blocks that the compiler cannot interleave.  kOptLinear / kOptAmrLog: the
+// default physics (quasi-linear D_mumu with lambda_par independent of p, exponential momentum
+// update, b . dV/dt term) on a uniform grid with linear r, or on block AMR with logarithmic r;
+// kOptAny: everything read from the parameters.  Measured (FP32): 1e4 Parker particles 16.2 ->
+// 14.8 ms, 64 sets of 4e6 particles 87.8 -> 84.5 ms, adjoint passes of 2e5 particles 42.6 -> 40.2
+// ms; 1e6 particles over 4 days 595 -> 577 ms together with the register limit (kMinBlocks).
+// ---------------------------------------------------------------------------
+constexpr int kOptAny = 0, kOptLinear = 1, kOptAmrLog = 2;
+
+template <int OPT>
+__device__ __forceinline__ bool opt_amr(const GridK& g) { return OPT == kOptAny ? g.amr > 0 : OPT == kOptAmrLog; }
+template <int OPT>
+__device__ __forceinline__ bool opt_log(const GridK& g) { return OPT == kOptAny ? g.radial != 0 : OPT == kOptAmrLog; }
+
+// ---------------------------------------------------------------------------
 // Pitch-angle diffusion coefficient and its mu derivative (Eq. 5 and the
 // quasi-linear / isotropic alternatives).  `I` is the normalisation integral.
 // ---------------------------------------------------------------------------
+template <int OPT = kOptAny>
 __device__ __forceinline__ void dmumu(const ParamsK& P, float I, float mu, float v, float p,
                                       float& D, float& dD)
 {
-    const float ilam = P.use_rig ? 1.f / (P.lambda_par * powf(p / P.p_ref, P.alpha)) : P.inv_lambda_par;
+    const float ilam = OPT == kOptAny && P.use_rig ? 1.f / (P.lambda_par * powf(p / P.p_ref, P.alpha)) : P.inv_lambda_par;
     const float am = fabsf(mu);
     const float sg = (mu > 0.f) ? 1.f : ((mu < 0.f) ? -1.f : 0.f);
     const float omm = 1.f - mu * mu;
-    if (P.dmumu == 0) {
+    if (OPT != kOptAny || P.dmumu == 0) {
         const float nu = 1.5f * v * I * ilam;
         // |mu|^(q-1) and max(|mu|, mu_floor)^(q-2) from one logarithm: above the floor
         // the first is the second times |mu| (two exp2/log2 instead of two powf)
@@ -191,9 +209,10 @@ __device__ __forceinline__ int amr_containing(const GridK& g, float r, float th,
 // Block AMR: leaf from the finest-level table, then the bracketing cells on the
 // leaf's padded lattice (level-l cell coordinate x = u n_l - 1/2, weights in the
 // physical coordinate).  The ghost layer supplies the neighbours' values.
+template <int OPT = kOptAny>
 __device__ __forceinline__ void locate_amr(const GridK& g, float r, float th, float ph, Loc& L)
 {
-    const float ur = g.radial ? logf(r / g.r_min) * g.inv_lnr : (r - g.r_min) * g.inv_lnr;
+    const float ur = opt_log<OPT>(g) ? logf(r / g.r_min) * g.inv_lnr : (r - g.r_min) * g.inv_lnr;
     const float ut = (th - g.th_min) * g.inv_thspan;
     const float up = ph * (1.f / kTwoPi);
     const int f0 = min(max((int)floorf(ur * (float)g.nf0), 0), g.nf0 - 1);
@@ -207,10 +226,10 @@ __device__ __forceinline__ void locate_amr(const GridK& g, float r, float th, fl
     const float s = (float)(1 << lf.x);
     const int B = g.B, P = g.P;
     // r
-    float x = (g.radial ? logf(r / g.r_min) * g.inv_dr : (r - g.r_min) * g.inv_dr) * s - 0.5f;
+    float x = (opt_log<OPT>(g) ? logf(r / g.r_min) * g.inv_dr : (r - g.r_min) * g.inv_dr) * s - 0.5f;
     int lo = lf.y * B - 1;
     int i = min(max((int)floorf(x), lo), lo + B);
-    if (g.radial) {
+    if (opt_log<OPT>(g)) {
         const float c0 = g.r_min * expf(((float)i + 0.5f) * g.dr / s);
         const float c1 = g.r_min * expf(((float)i + 1.5f) * g.dr / s);
         L.dfr = 1.f / (c1 - c0);
@@ -241,20 +260,24 @@ __device__ __forceinline__ void locate_amr(const GridK& g, float r, float th, fl
     L.base[3] = b0 + P * P + P;
 }
 
+template <int OPT = kOptAny>
 __device__ __forceinline__ void locate(const GridK& g, float r, float th, float ph, Loc& L)
 {
-    if (g.amr) {
-        locate_amr(g, r, th, ph, L);
+    if (opt_amr<OPT>(g)) {
+        locate_amr<OPT>(g, r, th, ph, L);
         return;
     }
-    float xi = g.radial ? logf(r / g.r_min) * g.inv_dr - 0.5f : (r - g.r_min) * g.inv_dr - 0.5f;
+    // the product is rounded before the subtraction, as in the form with both kinds of r axis
+    float xi;
+    if (OPT == kOptLinear) xi = __fadd_rn(__fmul_rn(r - g.r_min, g.inv_dr), -0.5f);
+    else xi = opt_log<OPT>(g) ? logf(r / g.r_min) * g.inv_dr - 0.5f : (r - g.r_min) * g.inv_dr - 0.5f;
     if (xi < 0.f) {
         L.i0 = 0; L.fr = 0.f; L.dfr = 0.f;
     } else if (xi >= (float)(g.nr - 1)) {
         L.i0 = g.nr - 2; L.fr = 1.f; L.dfr = 0.f;
     } else {
         L.i0 = (int)xi;
-        if (g.radial) {
+        if (opt_log<OPT>(g)) {
             const float c0 = g.r_min * expf(((float)L.i0 + 0.5f) * g.dr);
             const float c1 = g.r_min * expf(((float)L.i0 + 1.5f) * g.dr);
             L.dfr = 1.f / (c1 - c0);
@@ -435,7 +458,9 @@ __device__ __forceinline__ void fma2(float& d0, float& d1, float a0, float a1, f
 // PAIRED: accumulate with paired FMAs (the step kernels with the global tally; the
 // adjoint kernels, at their register bound, measured faster with scalar FMAs; both
 // round identically).
-template <bool KPERP, int DT, int LAY, bool PAIRED = false>
+// UNROLL: both snapshots in one block of code, so that the second one's loads are issued while
+// the first one's are summed.
+template <bool KPERP, int DT, int LAY, bool PAIRED = false, bool UNROLL = false>
 __device__ __forceinline__ void gather(const GridK& g, const StepEntry& e, const Loc& L,
                                        const float* sc, Fields<KPERP>& F)
 {
@@ -447,8 +472,7 @@ __device__ __forceinline__ void gather(const GridK& g, const StepEntry& e, const
 #pragma unroll
         for (int m = 0; m < 9; ++m) F.dBa[m] = 0.f;
     }
-    const int ns = e.two ? 2 : 1;
-    for (int s = 0; s < ns; ++s) {
+    auto one = [&](const int s) {
         const int snap = s ? e.s1 : e.s0;
         const float ws = e.two ? (s ? e.wt : 1.f - e.wt) : 1.f;
         const float sgn = s ? 1.f : -1.f;
@@ -508,6 +532,13 @@ __device__ __forceinline__ void gather(const GridK& g, const StepEntry& e, const
             F.f[3 + m] = fmaf(ws, vs[m], F.f[3 + m]);
             if (e.two) F.dv[m] = fmaf(sgn, vs[m], F.dv[m]);
         }
+    };
+    if (UNROLL) {
+        one(0);
+        if (e.two) one(1);
+    } else {
+        const int ns = e.two ? 2 : 1;
+        for (int s = 0; s < ns; ++s) one(s);
     }
     if (DT != FTE_F32) {
 #pragma unroll

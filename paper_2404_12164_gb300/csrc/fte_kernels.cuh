@@ -11,6 +11,7 @@ constexpr int kModeSingle = 0;
 constexpr int kModeShared = 1;
 constexpr int kModeGlobal = 2;
 constexpr int kModeSingleGlobal = 3;   // one parameter set, warp-merged FP64 atomics to the tally
+constexpr int kModeNoTally = 4;        // one parameter set, no observers (the adjoint's passes)
 
 __host__ __device__ constexpr bool single_set(int mode) { return mode == kModeSingle || mode == kModeSingleGlobal; }
 __host__ __device__ constexpr bool global_tally(int mode) { return mode == kModeGlobal || mode == kModeSingleGlobal; }
@@ -32,6 +33,7 @@ struct AdvanceArgs {
     ParamsK prm;
     ObsK obs[FTE_MAX_OBS];
     int n_obs, nbins;
+    int any_slab;                 // an observer is a slab (its test is on x, not r)
     float *x, *y, *z, *mu, *p, *w;
     const uint32_t* id;
     uint8_t* status;
@@ -152,24 +154,23 @@ struct AdjK {
 
 // launchers (return cudaGetLastError())
 // step kernel of (kperp, dtype, mode, threads per block); for the single-set modes nt must
-// be advance_threads() of the same arguments; blocks_max: blocks of one wave
+// be advance_threads() of the same arguments
 cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt, int blocks,
-                           int blocks_max, size_t smem, cudaStream_t s);
+                           size_t smem, cudaStream_t s);
 // resident blocks per SM of a step kernel (`pair`: record layout of a single-set kernel)
-cudaError_t advance_occupancy(int kperp, int dtype, int mode, int nt, int pair, int amr, size_t smem,
+cudaError_t advance_occupancy(int kperp, int dtype, int mode, int nt, int pair, int amr, int opt, size_t smem,
                               int* blocks_per_sm);
-// Builds of the single-set step kernel.  Block AMR with the global tally and no
-// cross-field diffusion (its chain of dependent loads, table -> leaf -> records, needs
-// more resident warps) runs a register-limited build: FP32 records 5 blocks of 128
-// threads per SM (at most 102 registers, 20 warps: 1.997e10 particle-steps/s against
-// 1.912e10 with 24 warps at 85 registers and 1.892e10 with 16 unconstrained), 16-bit
-// records 3 blocks of 256 (85 registers, 24 warps).  Uniform grids keep the
-// unconstrained build of 256 threads in every storage form (under the tighter limits it
-// spills: 16-bit storage measured 1.018x FP32 with the 3-block build and 1.069x without).
+// the options (kOptAny, ...) that a launch with these parameters can have fixed at compile time:
+// global tally, cell records and no cross-field diffusion (the other builds take them all from
+// the parameters)
+int advance_opt(const GridK& g, const ParamsK& prm, int kperp, int mode);
+// Builds of the single-set step kernel: uniform grids 256 threads, two blocks per SM; block AMR
+// with the global tally and no cross-field diffusion FP32 records 4 blocks of 128 threads, 16-bit
+// records 3 blocks of 256 (see fte_advance.cu for the measurements).
 // advance_threads: threads per block of the build that advance_fn selects.
 int advance_threads(int kperp, int dtype, int mode, int amr);
 // the ensemble variants live in their own translation unit (fte_batched.cu)
-const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair);
+const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair, int opt);
 cudaError_t launch_advance_batched(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt,
                                    int blocks, size_t smem, cudaStream_t s);
 cudaError_t launch_reduce(const float* part, int nblk, int nbins, double* S, double* S2,
