@@ -718,8 +718,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
             for (int k = 0; k < 2; ++k) {
                 ah[k].n_start = c0;
                 ah[k].n_end = (c0 + chunk < n_end) ? c0 + chunk : n_end;
-                FTE_CUDA(launch_sort(sh[k], hs[k]), "sort launch");
-                FTE_CUDA(cudaMemsetAsync(ah[k].fetch, 0, kFetchBytes, hs[k]), "fetch reset");
+                FTE_CUDA(launch_sort(sh[k], c0 == n_start, ah[k].fetch, kFetchSlots, hs[k]), "sort launch");
                 FTE_CUDA(launch_advance_timed(ah[k], kperp, mode, blocks, smem, hs[k], false), "step kernel launch");
             }
         }
@@ -731,8 +730,8 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
     for (long long c0 = n_start; c0 < n_end; c0 += chunk) {
         a.n_start = c0;
         a.n_end = (c0 + chunk < n_end) ? c0 + chunk : n_end;
-        if (sorting) FTE_CUDA(launch_sort(sa, st), "sort launch");
-        FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
+        if (sorting) FTE_CUDA(launch_sort(sa, c0 == n_start, a.fetch, kFetchSlots, st), "sort launch");
+        else FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
         FTE_CUDA(launch_advance_timed(a, kperp, mode, blocks, smem, st, cap != cudaStreamCaptureStatusNone),
                  "step kernel launch");
         if (nb && mode == kModeSingle)
@@ -1260,8 +1259,7 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
             for (int k = 0; k < 2; ++k) {
                 ah[k].n_start = c0;
                 ah[k].n_end = (c0 + cfg.steps < n_end) ? c0 + cfg.steps : n_end;
-                FTE_CUDA(launch_sort(sh[k], hs[k]), "sort launch");
-                FTE_CUDA(cudaMemsetAsync(ah[k].fetch, 0, kFetchBytes, hs[k]), "fetch reset");
+                FTE_CUDA(launch_sort(sh[k], c0 == n_start, ah[k].fetch, kFetchSlots, hs[k]), "sort launch");
                 FTE_CUDA(launch_advance(ah[k], bh[k], kperp, cfg.mode, cfg.nt, blocks, smem, hs[k]),
                          "step kernel launch");
             }
@@ -1274,8 +1272,8 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
     for (long long c0 = n_start; c0 < n_end; c0 += cfg.steps) {
         a.n_start = c0;
         a.n_end = (c0 + cfg.steps < n_end) ? c0 + cfg.steps : n_end;
-        if (sorting) FTE_CUDA(launch_sort(sa, st), "sort launch");
-        FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
+        if (sorting) FTE_CUDA(launch_sort(sa, c0 == n_start, a.fetch, kFetchSlots, st), "sort launch");
+        else FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
         FTE_CUDA(launch_advance(a, b, kperp, cfg.mode, cfg.nt, blocks, smem, st), "step kernel launch");
         if (cfg.mode == kModeShared && nb)
             FTE_CUDA(launch_reduce(a.part, blocks, reduce_bins, t->S, t->S2, t->C, st), "reduce launch");
@@ -1853,8 +1851,10 @@ fte_status fte_adjoint_forward(fte_particles* P, const fte_background* bg, const
                 a[h].n_start = c0;
                 a[h].n_end = c0 + sub < s1 ? c0 + sub : s1;
                 k[h].ckpt_on = c0 == s0;
-                if (sorting) FTE_CUDA(launch_sort(sa[h], hs[h]), "sort launch");
-                FTE_CUDA(cudaMemsetAsync(a[h].fetch, 0, kFetchBytes, hs[h]), "fetch reset");
+                if (sorting)
+                    FTE_CUDA(launch_sort(sa[h], c0 == n_start, a[h].fetch, kFetchSlots, hs[h]), "sort launch");
+                else
+                    FTE_CUDA(cudaMemsetAsync(a[h].fetch, 0, kFetchBytes, hs[h]), "fetch reset");
                 FTE_CUDA(launch_adjoint_forward(a[h], k[h], plan.L[h].fwd_blocks, hs[h]), "adjoint forward launch");
             }
         }
@@ -1955,14 +1955,16 @@ fte_status fte_adjoint_reverse(const fte_particles* P, const fte_background* bg,
                     sa[h].x = c; sa[h].y = c + n; sa[h].z = c + 2 * n; sa[h].mu = c + 3 * n;
                     sa[h].steps_min = k[h].c_start - n_start;
                     sa[h].order = orders[h] + (size_t)q * n;
-                    FTE_CUDA(launch_sort(sa[h], hs[h]), "sort launch");
+                    FTE_CUDA(launch_sort(sa[h], seg == plan.L[0].nseg - 1 && q == 0, a[h].fetch, kFetchSlots, hs[h]),
+                             "sort launch");
                     FTE_CUDA(cudaMemcpyAsync(counts[h] + q, sa[h].hist + sa[h].nb, sizeof(unsigned),
                                              cudaMemcpyDeviceToDevice, hs[h]),
                              "order count");
                     a[h].order = sa[h].order;
                     a[h].n_order = counts[h] + q;
+                } else {
+                    FTE_CUDA(cudaMemsetAsync(a[h].fetch, 0, kFetchBytes, hs[h]), "fetch reset");
                 }
-                FTE_CUDA(cudaMemsetAsync(a[h].fetch, 0, kFetchBytes, hs[h]), "fetch reset");
                 FTE_CUDA(launch_adjoint_replay(a[h], k[h], plan.L[h].rep_blocks, hs[h]), "adjoint replay launch");
             }
         }

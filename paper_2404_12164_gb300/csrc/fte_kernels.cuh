@@ -66,7 +66,7 @@ struct SortArgs {
     long long steps_min;
     unsigned long long n;
     unsigned* hist;               // bucket counts, then exclusive offsets; total at hist[nb]
-    unsigned* tiles;
+    unsigned* tiles;              // per tile of buckets: whether it holds particles
     int* key;
     int* rank;
     uint32_t* order;
@@ -201,7 +201,9 @@ cudaError_t launch_norm_derivs(int model, double q, double H, double eps, double
 // spatial ordering of the alive particles (fte_sort.cu)
 size_t sort_scratch_bytes(const GridK& g, unsigned long long n);
 void sort_carve(const GridK& g, unsigned long long n, char* p, SortArgs* a);
-cudaError_t launch_sort(const SortArgs& a, cudaStream_t s);
+// `first`: the scratch holds anything (first reordering of a call); otherwise it is as the last
+// launch_sort with the same arguments left it.  fetch: n_fetch work counters to reset.
+cudaError_t launch_sort(const SortArgs& a, bool first, unsigned long long* fetch, int n_fetch, cudaStream_t s);
 // block AMR set-up (fte_amr.cu): status[0] malformed leaves, [1] overlaps,
 // [2] uncovered finest blocks, [3] 2:1 nesting violations
 cudaError_t launch_amr_table(const GridK& g, int* table, unsigned* status, cudaStream_t s);

@@ -58,6 +58,10 @@ __device__ __forceinline__ int bucket_of(const GridK& g, float x, float y, float
 // measured best: four halve the particles per bucket for a smaller gain.
 constexpr int kMuBins = 2;
 
+constexpr int kScanThreads = 256;
+constexpr int kScanItems = 16;
+constexpr int kScanTile = kScanThreads * kScanItems;
+
 __global__ void __launch_bounds__(256) key_kernel(const SortArgs a)
 {
     const unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -68,16 +72,23 @@ __global__ void __launch_bounds__(256) key_kernel(const SortArgs a)
         if (a.mu) mb = min(max((int)((a.mu[i] + 1.f) * (0.5f * kMuBins)), 0), kMuBins - 1);
         key = bucket_of(a.g, a.x[i], a.y[i], a.z[i]) * kMuBins + mb;
         rank = (int)atomicAdd(a.hist + key, 1u);
+        if (rank == 0) a.tiles[key / kScanTile] = 1u;
     }
     a.key[i] = key;
     a.rank[i] = rank;
 }
 
-// three-phase exclusive scan of hist[0..nb) into hist, total into hist[nb]
-constexpr int kScanThreads = 1024;
-constexpr int kScanItems = 4;
-constexpr int kScanTile = kScanThreads * kScanItems;
-
+// Bucket counts -> first entry of every bucket in the order list, in one pass over the tiles of
+// kScanTile buckets that hold particles: each block scans its tile and takes the tile's place in
+// the list from the running total hist[nb] (buckets stay in order within a tile; which tile comes
+// first does not matter to any result).  Most tiles are empty - the particles sit in a few per
+// cent of the grid - so a tile's flag, set by its first particle, spares reading it, and before the
+// next reordering only the flagged tiles are zeroed again.  The whole histogram (22 MB on a 512 x
+// 60 x 180 grid, 0.2 GB on 11,296 AMR leaves) used to be cleared, read, and read and written once
+// per reordering, in a clear and three scan launches: 38 us for the 22 MB against 9 us now, 0.24 ms
+// against 24 us for the 0.2 GB (1e6 particles over 4 days 580 -> 543 ms, 3e5 in BF16 25.8 -> 23.7
+// ms, 9e4 on 3-level AMR, 90 steps, 2.0 -> 1.0 ms).  The work counters of the step kernel that
+// follows are reset here too.
 __device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned* sh, unsigned* total)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -89,71 +100,76 @@ __device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned* s
     }
     if (lane == 31) sh[wid] = x;
     __syncthreads();
-    if (wid == 0) {
-        unsigned s = (lane < (int)(blockDim.x >> 5)) ? sh[lane] : 0u;
+    unsigned off = 0, sum = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        sh[lane] = s;
+    for (int w = 0; w < kScanThreads / 32; ++w) {
+        const unsigned t = sh[w];
+        if (w < wid) off += t;
+        sum += t;
     }
-    __syncthreads();
-    const unsigned warp_off = wid ? sh[wid - 1] : 0u;
-    *total = sh[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return warp_off + x - v;
+    *total = sum;
+    return off + x - v;
 }
 
-__global__ void __launch_bounds__(kScanThreads) tile_sum_kernel(const unsigned* hist, int nb, unsigned* tiles)
+__global__ void __launch_bounds__(kScanThreads) scan_kernel(unsigned* hist, int nb, const unsigned* tiles,
+                                                            unsigned long long* fetch, int n_fetch)
 {
-    __shared__ unsigned sh[32];
-    const long long base = (long long)blockIdx.x * kScanTile + threadIdx.x * kScanItems;
-    unsigned s = 0;
-#pragma unroll
-    for (int q = 0; q < kScanItems; ++q)
-        if (base + q < nb) s += hist[base + q];
-    unsigned total;
-    block_exclusive_scan(s, sh, &total);
-    if (threadIdx.x == 0) tiles[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(kScanThreads) tile_offsets_kernel(unsigned* tiles, int ntiles)
-{
-    // one block: exclusive scan of the tile sums, in chunks of blockDim.x
-    __shared__ unsigned sh[32];
-    unsigned carry = 0;
-    for (int b0 = 0; b0 < ntiles; b0 += kScanThreads) {
-        const int t = b0 + threadIdx.x;
-        const unsigned v = t < ntiles ? tiles[t] : 0u;
-        unsigned total;
-        const unsigned ex = block_exclusive_scan(v, sh, &total);
-        if (t < ntiles) tiles[t] = carry + ex;
-        carry += total;
-    }
-    if (threadIdx.x == 0) tiles[ntiles] = carry;
-}
-
-__global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(unsigned* hist, int nb, const unsigned* tiles,
-                                                                 int ntiles)
-{
-    __shared__ unsigned sh[32];
+    __shared__ unsigned sh[kScanThreads / 32], s_base;
+    if (blockIdx.x == 0)
+        for (int q = threadIdx.x; q < n_fetch; q += kScanThreads) fetch[q] = 0ULL;
+    if (tiles[blockIdx.x] == 0u) return;
     const long long base = (long long)blockIdx.x * kScanTile + threadIdx.x * kScanItems;
     unsigned v[kScanItems];
-    unsigned s = 0;
+    unsigned sum = 0;
+    const bool whole = base + kScanItems <= nb;     // base is a multiple of 16 entries: 16-byte accesses
+    uint4* h4 = reinterpret_cast<uint4*>(hist + base);
+    if (whole) {
 #pragma unroll
-    for (int q = 0; q < kScanItems; ++q) {
-        v[q] = (base + q < nb) ? hist[base + q] : 0u;
-        s += v[q];
+        for (int q = 0; q < kScanItems / 4; ++q) {
+            const uint4 t = h4[q];
+            v[4 * q] = t.x; v[4 * q + 1] = t.y; v[4 * q + 2] = t.z; v[4 * q + 3] = t.w;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < kScanItems; ++q) v[q] = (base + q < nb) ? hist[base + q] : 0u;
     }
+#pragma unroll
+    for (int q = 0; q < kScanItems; ++q) sum += v[q];
     unsigned total;
-    unsigned run = tiles[blockIdx.x] + block_exclusive_scan(s, sh, &total);
+    const unsigned ex = block_exclusive_scan(sum, sh, &total);
+    if (threadIdx.x == 0) s_base = atomicAdd(hist + nb, total);
+    __syncthreads();
+    unsigned run = s_base + ex;
 #pragma unroll
     for (int q = 0; q < kScanItems; ++q) {
-        if (base + q < nb) hist[base + q] = run;
-        run += v[q];
+        const unsigned t = v[q];
+        v[q] = run;
+        run += t;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) hist[nb] = tiles[ntiles];
+    if (whole) {
+#pragma unroll
+        for (int q = 0; q < kScanItems / 4; ++q)
+            h4[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < kScanItems; ++q)
+            if (base + q < nb) hist[base + q] = v[q];
+    }
+}
+
+// Zeroes the flagged tiles and their flags, and the total.
+__global__ void __launch_bounds__(kScanThreads) clear_kernel(unsigned* hist, int nb, unsigned* tiles)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0) hist[nb] = 0u;
+    if (tiles[blockIdx.x] == 0u) return;
+    const long long base = (long long)blockIdx.x * kScanTile;
+#pragma unroll
+    for (int q = 0; q < kScanItems; ++q) {
+        const long long b = base + q * kScanThreads + threadIdx.x;
+        if (b < nb) hist[b] = 0u;
+    }
+    __syncthreads();                  // every thread has read the flag
+    if (threadIdx.x == 0) tiles[blockIdx.x] = 0u;
 }
 
 __global__ void __launch_bounds__(256) scatter_kernel(const SortArgs a)
@@ -194,15 +210,17 @@ void sort_carve(const GridK& g, unsigned long long n, char* p, SortArgs* a)
     a->ntiles = (int)ntiles;
 }
 
-cudaError_t launch_sort(const SortArgs& a, cudaStream_t s)
+cudaError_t launch_sort(const SortArgs& a, bool first, unsigned long long* fetch, int n_fetch, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(a.hist, 0, (size_t)(a.nb + 1) * 4, s);
-    if (e != cudaSuccess) return e;
+    if (first) {        // the workspace holds anything: histogram, total and flags lie side by side
+        const cudaError_t e = cudaMemsetAsync(a.hist, 0, (char*)(a.tiles + a.ntiles) - (char*)a.hist, s);
+        if (e != cudaSuccess) return e;
+    } else {
+        clear_kernel<<<a.ntiles, kScanThreads, 0, s>>>(a.hist, a.nb, a.tiles);
+    }
     const unsigned blocks = (unsigned)((a.n + 255) / 256);
     if (blocks) key_kernel<<<blocks, 256, 0, s>>>(a);
-    tile_sum_kernel<<<a.ntiles, kScanThreads, 0, s>>>(a.hist, a.nb, a.tiles);
-    tile_offsets_kernel<<<1, kScanThreads, 0, s>>>(a.tiles, a.ntiles);
-    tile_scan_kernel<<<a.ntiles, kScanThreads, 0, s>>>(a.hist, a.nb, a.tiles, a.ntiles);
+    scan_kernel<<<a.ntiles, kScanThreads, 0, s>>>(a.hist, a.nb, a.tiles, fetch, n_fetch);
     if (blocks) scatter_kernel<<<blocks, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
