@@ -320,10 +320,8 @@ cudaError_t launch_reduce(const float* part, int nblk, int nbins, double* S, dou
 // time weight, and the time bin of every observer (rounded operations, no
 // contraction, so that edges fall exactly where the definition puts them).
 // ---------------------------------------------------------------------------
-__global__ void step_table_kernel(const StepTableArgs a)
+__device__ __forceinline__ void step_table_entry(const StepTableArgs& a, long long k)
 {
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= a.count) return;
     const long long n = a.n0 + k;
     const double t = __dadd_rn(a.t0, __dmul_rn((double)n, a.dt));
     StepEntry e;
@@ -367,101 +365,131 @@ __global__ void step_table_kernel(const StepTableArgs a)
     a.tab[k] = e;
 }
 
-cudaError_t launch_step_table(const StepTableArgs& a, cudaStream_t s)
-{
-    const int blocks = (int)((a.count + 255) / 256);
-    if (blocks > 0) step_table_kernel<<<blocks, 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------------------
 // Normalisation of D_mumu from lambda_par: I (quasi-linear) or J (Eq. 5), by
-// composite Simpson in FP64 after mu = s^3; 1 for the isotropic form.  Stage 1:
-// one node per thread, block sums in a fixed tree order; stage 2: one thread adds
-// the block sums in order.
+// composite Simpson in FP64 after mu = s^3; 1 for the isotropic form, one set per
+// blockIdx.y.  The nodes are summed in trees of 256 and the trees' sums in order.
+// A tree is spread over four blocks by node index mod 4 (its last two levels, which
+// add the four residue classes, come in the second kernel): 16,385 FP64 powers on 260
+// blocks of 64 threads keep every SM's slow FP64 unit busy (6.8 us), where 65 blocks of
+// 256 ran on 65 SMs (11.4 us).
 // ---------------------------------------------------------------------------
 constexpr int kNormIntervals = 16384;
-constexpr int kNormThreads = 256;
-constexpr int kNormBlocks = kNormIntervals / kNormThreads + 1;   // nodes 0 .. kNormIntervals
-static_assert(kNormBlocks <= kNormPartials, "norm partials");
+constexpr int kNormTree = 256;
+constexpr int kNormTrees = kNormIntervals / kNormTree + 1;   // nodes 0 .. kNormIntervals
+constexpr int kNormSplit = 4;
+constexpr int kNormThreads = kNormTree / kNormSplit;
+static_assert(kNormTrees * kNormSplit <= kNormPartials, "norm partials");
 
-__global__ void __launch_bounds__(kNormThreads) norm_partial_kernel(int model, double q, double H,
-                                                                    double eps, double* part)
+template <int NS>
+struct NormArgs {
+    int model;
+    double q[NS], H[NS], eps[NS];
+    double* part;                 // [set][kNormPartials]
+};
+
+template <int NS>
+__global__ void __launch_bounds__(kNormThreads) norm_partial_kernel(const NormArgs<NS> a)
 {
-    __shared__ double sh[kNormThreads];
-    const int i = blockIdx.x * kNormThreads + threadIdx.x;
+    __shared__ double upper[32];
+    const int s = NS > 1 ? blockIdx.y : 0;
+    const int tree = blockIdx.x / kNormSplit, c = blockIdx.x % kNormSplit, u = threadIdx.x;
+    const int i = tree * kNormTree + u * kNormSplit + c;
     double f = 0.0;
-    if (model != 2 && i <= kNormIntervals) {
+    if (a.model != 2 && i <= kNormIntervals) {
         const double h = 1.0 / kNormIntervals;
-        const double s = i * h;
-        const double m = s * s * s;
-        const double den = (model == 0) ? pow(m, q - 1.0) + H : m / (1.0 + m) + eps;
+        const double x = i * h;
+        const double m = x * x * x;
+        const double den = (a.model == 0) ? pow(m, a.q[s] - 1.0) + a.H[s] : m / (1.0 + m) + a.eps[s];
         const double wgt = (i == 0 || i == kNormIntervals) ? 1.0 : ((i & 1) ? 4.0 : 2.0);
-        f = wgt * 3.0 * s * s * (1.0 - m * m) / den;
+        f = wgt * 3.0 * x * x * (1.0 - m * m) / den;
     }
-    sh[threadIdx.x] = f;
+    // the tree's levels above the four residue classes: node t adds node t + 128, 64, .. 4
+    if (u >= 32) upper[u - 32] = f;
     __syncthreads();
-    for (int o = kNormThreads / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+    if (u >= 32) return;
+    f += upper[u];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) f += __shfl_down_sync(0xffffffffu, f, o);
+    if (u == 0) a.part[(size_t)s * kNormPartials + blockIdx.x] = f;
 }
 
-__global__ void norm_final_kernel(int model, const double* part, double* out)
+// What the step kernels read besides the particles: the step table (blocks 0 .. table_blocks - 1)
+// and the normalisation integrals from their partial sums (one further block), in one launch
+// (5.3 us; 5.4 + 4.1 us in two).
+__global__ void __launch_bounds__(256) setup_kernel(const StepTableArgs a, int table_blocks, int model, int n_sets,
+                                                    const double* part, double* out)
 {
-    double acc = 0.0;
-    for (int b = 0; b < kNormBlocks; ++b) acc += part[b];
-    out[0] = (model == 2) ? 1.0 : acc / (3.0 * kNormIntervals);
-}
-
-// one block row per set (blockIdx.y), same quadrature
-__global__ void __launch_bounds__(kNormThreads) norm_sets_partial_kernel(int model, const NormSets ns,
-                                                                         double* part)
-{
-    const int s = blockIdx.y;
-    __shared__ double sh[kNormThreads];
-    const int i = blockIdx.x * kNormThreads + threadIdx.x;
-    double f = 0.0;
-    if (model != 2 && i <= kNormIntervals) {
-        const double h = 1.0 / kNormIntervals;
-        const double u = i * h;
-        const double m = u * u * u;
-        const double den = (model == 0) ? pow(m, ns.q[s] - 1.0) + ns.H[s] : m / (1.0 + m) + ns.eps[s];
-        const double wgt = (i == 0 || i == kNormIntervals) ? 1.0 : ((i & 1) ? 4.0 : 2.0);
-        f = wgt * 3.0 * u * u * (1.0 - m * m) / den;
+    if ((int)blockIdx.x < table_blocks) {
+        const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        if (k < a.count) step_table_entry(a, k);
+        return;
     }
-    sh[threadIdx.x] = f;
+    __shared__ double tree[FTE_MAX_SETS * kNormTrees];
+    for (int k = threadIdx.x; k < n_sets * kNormTrees; k += blockDim.x) {
+        const double* p = part + (size_t)(k / kNormTrees) * kNormPartials + (k % kNormTrees) * kNormSplit;
+        tree[k] = (p[0] + p[2]) + (p[1] + p[3]);       // the last two levels of the tree
+    }
     __syncthreads();
-    for (int o = kNormThreads / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
+    if ((int)threadIdx.x < n_sets) {
+        double acc = 0.0;
+        for (int b = 0; b < kNormTrees; ++b) acc += tree[threadIdx.x * kNormTrees + b];
+        out[threadIdx.x] = (model == 2) ? 1.0 : acc / (3.0 * kNormIntervals);
     }
-    if (threadIdx.x == 0) part[(size_t)s * kNormPartials + blockIdx.x] = sh[0];
 }
 
-__global__ void norm_sets_final_kernel(int model, int n_sets, const double* part, double* out)
+static cudaError_t launch_second(const StepTableArgs* ta, int model, int n_sets, const double* part, double* out,
+                                 cudaStream_t s)
 {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n_sets) return;
-    double acc = 0.0;
-    for (int b = 0; b < kNormBlocks; ++b) acc += part[(size_t)s * kNormPartials + b];
-    out[s] = (model == 2) ? 1.0 : acc / (3.0 * kNormIntervals);
-}
-
-cudaError_t launch_norm_sets(int model, const NormSets& ns, int n_sets, double* out, double* part,
-                             cudaStream_t s)
-{
-    norm_sets_partial_kernel<<<dim3(kNormBlocks, n_sets), kNormThreads, 0, s>>>(model, ns, part);
-    norm_sets_final_kernel<<<1, 64, 0, s>>>(model, n_sets, part, out);
+    StepTableArgs none = {};
+    if (!ta) ta = &none;
+    const int tb = (int)((ta->count + 255) / 256), blocks = tb + (n_sets > 0 ? 1 : 0);
+    if (blocks > 0) setup_kernel<<<blocks, 256, 0, s>>>(*ta, tb, model, n_sets, part, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_norm(int model, double q, double H, double eps, double* out, double* part,
-                        cudaStream_t s)
+cudaError_t launch_step_table(const StepTableArgs& a, cudaStream_t s)
 {
-    norm_partial_kernel<<<kNormBlocks, kNormThreads, 0, s>>>(model, q, H, eps, part);
-    norm_final_kernel<<<1, 1, 0, s>>>(model, part, out);
+    return launch_second(&a, 2, 0, nullptr, nullptr, s);
+}
+
+cudaError_t launch_setup(int model, double q, double H, double eps, double* out, double* part,
+                         const StepTableArgs* ta, cudaStream_t s)
+{
+    const NormArgs<1> a = {model, {q}, {H}, {eps}, part};
+    norm_partial_kernel<1><<<kNormTrees * kNormSplit, kNormThreads, 0, s>>>(a);
+    return launch_second(ta, model, 1, part, out, s);
+}
+
+cudaError_t launch_setup_sets(int model, const NormSets& ns, int n_sets, double* out, double* part,
+                              const StepTableArgs* ta, cudaStream_t s)
+{
+    NormArgs<FTE_MAX_SETS> a;
+    a.model = model;
+    a.part = part;
+    for (int k = 0; k < FTE_MAX_SETS; ++k) { a.q[k] = ns.q[k]; a.H[k] = ns.H[k]; a.eps[k] = ns.eps[k]; }
+    norm_partial_kernel<FTE_MAX_SETS><<<dim3(kNormTrees * kNormSplit, n_sets), kNormThreads, 0, s>>>(a);
+    return launch_second(ta, model, n_sets, part, out, s);
+}
+
+// ---------------------------------------------------------------------------
+// Zeroes up to six arrays of 8-byte values in one launch (the tally and its ledger: 3 us instead
+// of six clears of about 1.5 us each).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) zero_kernel(const ZeroArgs a)
+{
+    const size_t step = (size_t)gridDim.x * blockDim.x, first = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        for (size_t i = first; i < a.n[k]; i += step) a.p[k][i] = 0ULL;
+}
+
+cudaError_t launch_zero(const ZeroArgs& a, cudaStream_t s)
+{
+    size_t most = 1;
+    for (int k = 0; k < 6; ++k) most = a.n[k] > most ? a.n[k] : most;
+    const size_t blocks = (most + 1023) / 1024;
+    zero_kernel<<<(unsigned)(blocks < 1216 ? blocks : 1216), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -503,15 +503,14 @@ fte_status fte_tally_reset(const fte_tally_buf* t, void* stream)
     if (s != FTE_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     nb *= (size_t)(t->n_sets > 1 ? t->n_sets : 1);
-    if (nb) {
-        FTE_CUDA(cudaMemsetAsync(t->S, 0, nb * sizeof(double), st), "memset S");
-        FTE_CUDA(cudaMemsetAsync(t->S2, 0, nb * sizeof(double), st), "memset S2");
-        FTE_CUDA(cudaMemsetAsync(t->C, 0, nb * sizeof(unsigned long long), st), "memset C");
-    }
-    if (t->S_class && nb)
-        FTE_CUDA(cudaMemsetAsync(t->S_class, 0, nb * FTE_NCLASS * sizeof(double), st), "memset S_class");
-    FTE_CUDA(cudaMemsetAsync(t->ledger_w, 0, FTE_LEDGER * sizeof(double), st), "memset ledger");
-    FTE_CUDA(cudaMemsetAsync(t->ledger_n, 0, FTE_LEDGER * sizeof(unsigned long long), st), "memset ledger");
+    ZeroArgs z;
+    memset(&z, 0, sizeof(z));
+    auto set = [&](int k, void* p, size_t n) { z.p[k] = (unsigned long long*)p; z.n[k] = n; };
+    if (nb) { set(0, t->S, nb); set(1, t->S2, nb); set(2, t->C, nb); }
+    if (t->S_class && nb) set(3, t->S_class, nb * FTE_NCLASS);
+    set(4, t->ledger_w, FTE_LEDGER);
+    set(5, t->ledger_n, FTE_LEDGER);
+    FTE_CUDA(launch_zero(z, st), "tally reset");
     return FTE_OK;
 }
 
@@ -614,9 +613,6 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
     cudaStream_t st = (cudaStream_t)stream;
 
     double* norm = (double*)(w + L.off_norm);
-    FTE_CUDA(launch_norm(prm->dmumu, prm->q, prm->H, prm->eps, norm, (double*)(w + L.off_npart), st),
-             "norm launch");
-
     StepTableArgs ta;
     memset(&ta, 0, sizeof(ta));
     ta.tab = (StepEntry*)(w + L.off_table);
@@ -627,7 +623,8 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
     for (int o = 0; o < t->n_obs; ++o) {
         ta.ot[o].t_lo = t->obs[o].t_lo; ta.ot[o].t_hi = t->obs[o].t_hi; ta.ot[o].nt = t->obs[o].nt;
     }
-    FTE_CUDA(launch_step_table(ta, st), "step table launch");
+    FTE_CUDA(launch_setup(prm->dmumu, prm->q, prm->H, prm->eps, norm, (double*)(w + L.off_npart), &ta, st),
+             "set-up launch");
 
     AdvanceArgs a;
     memset(&a, 0, sizeof(a));
@@ -971,8 +968,9 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
     // scratch layout: fetch counter, normalisation, the time table of one
     // launch, then per-block partial histograms
     const int kperp = prm->lambda_perp > 0.0 ? 1 : 0;
-    const size_t off_fetch = 0, off_norm = 64, off_npart = 128;
-    const size_t off_table = off_npart + kNormPartials * sizeof(double);
+    // (the normalisation's partial sums are used up before the first table is written in their place)
+    const size_t off_fetch = 0, off_norm = 64, off_table = 128 + 128 * sizeof(double), off_npart = off_table;
+    static_assert(kNormPartials * sizeof(double) <= (size_t)kChunkSteps * sizeof(StepEntry), "norm scratch");
     const size_t off_part = (off_table + (size_t)kChunkSteps * sizeof(StepEntry) + 255) & ~(size_t)255;
     const size_t part_block = 3 * sizeof(float) * (nb ? nb : 1);
     const int sms = device_sms(device);
@@ -992,7 +990,7 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
 
     cudaStream_t st = (cudaStream_t)stream;
     double* norm = (double*)(w + off_norm);
-    FTE_CUDA(launch_norm(prm->dmumu, prm->q, prm->H, prm->eps, norm, (double*)(w + off_npart), st),
+    FTE_CUDA(launch_setup(prm->dmumu, prm->q, prm->H, prm->eps, norm, (double*)(w + off_npart), nullptr, st),
              "norm launch");
 
     AdvanceArgs a;
@@ -1152,7 +1150,6 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
     memset(&ns, 0, sizeof(ns));
     for (int k = 0; k < n_sets; ++k) { ns.q[k] = sets[k].q; ns.H[k] = sets[k].H; ns.eps[k] = sets[k].eps; }
     double* norm = (double*)(w + L.off_norm);
-    FTE_CUDA(launch_norm_sets(prm->dmumu, ns, n_sets, norm, (double*)(w + L.off_npart), st), "norm launch");
 
     StepTableArgs ta;
     memset(&ta, 0, sizeof(ta));
@@ -1164,7 +1161,7 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
     for (int o = 0; o < t->n_obs; ++o) {
         ta.ot[o].t_lo = t->obs[o].t_lo; ta.ot[o].t_hi = t->obs[o].t_hi; ta.ot[o].nt = t->obs[o].nt;
     }
-    FTE_CUDA(launch_step_table(ta, st), "step table launch");
+    FTE_CUDA(launch_setup_sets(prm->dmumu, ns, n_sets, norm, (double*)(w + L.off_npart), &ta, st), "set-up launch");
 
     AdvanceArgs a;
     memset(&a, 0, sizeof(a));
@@ -1644,10 +1641,10 @@ fte_status adj_args(const fte_particles* P, const fte_background* bg, const fte_
     ta.n_snap = bg->grid.n_snap; ta.periodic = bg->grid.periodic; ta.ring = bg->grid.ring;
     ta.t_snap0 = bg->grid.t_snap0; ta.dt_snap = bg->grid.dt_snap;
     if (setup) {
-        FTE_CUDA(launch_norm(prm->dmumu, prm->q, prm->H, prm->eps, norm, (double*)(w + L.off_npart), st), "norm launch");
+        FTE_CUDA(launch_setup(prm->dmumu, prm->q, prm->H, prm->eps, norm, (double*)(w + L.off_npart),
+                              nsteps > 0 ? &ta : nullptr, st), "set-up launch");
         FTE_CUDA(launch_norm_derivs(prm->dmumu, prm->q, prm->H, prm->eps, normd, (double*)(w + L.off_ndpart), st),
                  "norm derivative launch");
-        if (nsteps > 0) FTE_CUDA(launch_step_table(ta, st), "step table launch");
     }
     memset(a, 0, sizeof(*a));
     a->obs[0].dr = -1.f;               // no observers

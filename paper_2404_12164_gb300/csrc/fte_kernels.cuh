@@ -176,13 +176,19 @@ cudaError_t launch_advance_batched(const AdvanceArgs& a, const BatchArgs& b, int
 cudaError_t launch_reduce(const float* part, int nblk, int nbins, double* S, double* S2,
                           unsigned long long* C, cudaStream_t s);
 cudaError_t launch_step_table(const StepTableArgs& a, cudaStream_t s);
-// normalisation integral; `part` holds kNormPartials doubles of scratch
-constexpr int kNormPartials = 128;
-cudaError_t launch_norm(int model, double q, double H, double eps, double* out, double* part,
-                        cudaStream_t s);
+// normalisation integral and step table (ta may be NULL); `part` holds kNormPartials doubles of scratch
+constexpr int kNormPartials = 272;
+cudaError_t launch_setup(int model, double q, double H, double eps, double* out, double* part,
+                         const StepTableArgs* ta, cudaStream_t s);
 // the same for n_sets sets at once: out[s], scratch part[n_sets][kNormPartials]
-cudaError_t launch_norm_sets(int model, const NormSets& ns, int n_sets, double* out, double* part,
-                             cudaStream_t s);
+cudaError_t launch_setup_sets(int model, const NormSets& ns, int n_sets, double* out, double* part,
+                              const StepTableArgs* ta, cudaStream_t s);
+// n[k] 8-byte values at p[k] set to zero
+struct ZeroArgs {
+    unsigned long long* p[6];
+    size_t n[6];
+};
+cudaError_t launch_zero(const ZeroArgs& a, cudaStream_t s);
 cudaError_t launch_tally_out(const double* S, const double* S2, const unsigned long long* C,
                              const ObsOut& ob, int kind, double* out, cudaStream_t s);
 cudaError_t launch_convolve(const double* S, const ObsOut& ob, int kind, const double* src, double* out,
