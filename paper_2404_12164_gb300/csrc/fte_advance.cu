@@ -118,16 +118,22 @@ cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, 
                                 near);
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {(void*)&a, (void*)&b};
-    // A pool that is not reordered is launched in blocks of one warp, which spread evenly over the
-    // SMs: 1e4 particles in blocks of 256 occupy 40 of 152 SMs with 8 warps each, in blocks of 32
-    // every SM with 2, and a step's latency falls with the warps it shares an SM with (1e4
-    // particles x 8640 steps 19.1 -> 17.4 ms, 2000 x 200 0.54 -> 0.50 ms); 1.3e5 particles, two
-    // per thread, are 248 blocks of 256, two on 96 SMs and one on 56.  Global tally only: a block
-    // of the shared-memory tally carries a whole histogram.
-    if (mode == kModeSingleGlobal && !a.order) {
-        const unsigned long long warps = (a.n_particles + 31) / 32, given = (unsigned long long)blocks * (nt / 32);
-        blocks = (int)(warps < given ? warps : given);
-        nt = 32;
+    // The global-tally kernels share nothing within a block, so blocks only decide how warps
+    // spread over the SMs.  A pool that is not reordered goes in blocks of one warp: 1e4 particles
+    // in blocks of 256 occupy 40 of 152 SMs with 8 warps each, in blocks of 32 every SM with 2, and
+    // a step's latency falls with the warps it shares an SM with (1e4 particles x 8640 steps 19.1
+    // -> 17.4 ms, 2000 x 200 0.54 -> 0.50 ms); 1.3e5 particles, two per thread, are 248 blocks of
+    // 256, two on 96 SMs and one on 56.  A reordered pool launches one wave in blocks of 64: when
+    // few particles are left alive and the surplus blocks leave at once (see advance_kernel), those
+    // that stay are spread as evenly (1e6 particles over 4 days, 4.6e4 alive at the end: 543 ms in
+    // blocks of 256, 531 of 128, 530 of 64, 528 of 32; 1.2e5 with cross-field diffusion 929 -> 910
+    // us).  A block of the shared-memory tally carries a whole histogram and stays as it is.
+    if (mode == kModeSingleGlobal) {
+        const int small = a.order ? 64 : 32;
+        const unsigned long long need = (a.n_particles + small - 1) / small,
+                                 given = (unsigned long long)blocks * (nt / small);
+        blocks = (int)(a.order || need >= given ? given : need);
+        nt = small;
     }
     return cudaLaunchKernel(fn, dim3(blocks), dim3(nt), args, smem, s);
 }

@@ -377,9 +377,9 @@ __global__ void __launch_bounds__(NT, single_set(MODE) ? MINB : 512 / NT) advanc
     // counter.  A pool launched alone keeps all blocks: there the freed slots would stay idle.
     unsigned fetch_slots = a.fetch_slots;
     if (MODE == kModeSingleGlobal && a.order && a.compact) {
-        if (n_work < (unsigned long long)gridDim.x * NT) {
+        if (n_work < (unsigned long long)gridDim.x * blockDim.x) {
             fetch_slots = 0;
-            if (blockIdx.x >= (n_work + NT - 1) / NT) return;
+            if (blockIdx.x >= (n_work + blockDim.x - 1) / blockDim.x) return;
         }
     }
     unsigned long long nsteps = 0, noor = 0;
