@@ -458,10 +458,10 @@ def run_gpu(args):
                                                                           adjoint["t_c"]))
 
     roofline = roofline_record(intervals, total_steps // ws, ALG_BYTES, l1, l2_gbs, measured_traffic(args.layout))
-    # our kernels per timed step: inject, and per advance call the two normalisation
-    # kernels and the step table, then per launch chunk the step kernel, (with the
-    # shared-memory tally) the partial-histogram reduction and (with reordering) the
-    # five sort kernels
+    # our kernels per timed step: tally reset and inject, and per advance call the normalisation's
+    # partial sums and the set-up (its final sums and the step table), then per launch chunk the
+    # step kernel, (with the shared-memory tally) the partial-histogram reduction and (with
+    # reordering) the key, scan and scatter kernels and, from a call's second chunk on, the clear
     # a pool of at least one wave of threads (at most 3 blocks of 256 per SM) is advanced as
     # two halves, each with its own reordering and launches (global tally, reordering on)
     wave = torch.cuda.get_device_properties(local).multi_processor_count * 3 * 256
@@ -469,9 +469,11 @@ def run_gpu(args):
 
     def kernels_per_call(s):
         chunk = min(w.params.sort_every, CHUNK) if w.params.sort_every > 0 else CHUNK
-        per_chunk = 1 + (1 if w.params.tally_layout == "shared" else 0) + (5 if w.params.sort_every > 0 else 0)
-        return 3 + math.ceil(s / chunk) * per_chunk * halves
-    launches_per_step = 1 + sum(kernels_per_call(min(CHUNK, n_steps - c)) for c in range(0, n_steps, CHUNK))
+        chunks = math.ceil(s / chunk)
+        per_chunk = 1 + (1 if w.params.tally_layout == "shared" else 0)
+        sort = 4 * chunks - 1 if w.params.sort_every > 0 else 0
+        return 2 + (chunks * per_chunk + sort) * halves
+    launches_per_step = 2 + sum(kernels_per_call(min(CHUNK, n_steps - c)) for c in range(0, n_steps, CHUNK))
     result = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,

@@ -625,14 +625,14 @@ cudaError_t adjoint_blocks(int dtype, int pair, int kind, int* blocks_per_sm)
 static cudaError_t launch_adj(int kind, const AdvanceArgs& a, const AdjK& k, int blocks, cudaStream_t s)
 {
     void* args[] = {(void*)&a, (void*)&k};
-    // a pool that is not reordered goes in blocks of one warp, as in launch_advance (2e4 particles,
-    // 400 steps forward and back: 6.32 -> 6.04 ms)
-    if (!a.order) {
-        const unsigned long long warps = (a.n_particles + 31) / 32, given = (unsigned long long)blocks * 8;
-        return cudaLaunchKernel(adj_fn(kind, a.g.dtype, a.g.pair, adjoint_opt(a.g, a.prm)),
-                                dim3((unsigned)(warps < given ? warps : given)), dim3(32), args, 0, s);
-    }
-    return cudaLaunchKernel(adj_fn(kind, a.g.dtype, a.g.pair, adjoint_opt(a.g, a.prm)), dim3(blocks), dim3(256), args, 0, s);
+    const int opt = adjoint_opt(a.g, a.prm);
+    // Blocks only decide how warps spread over the SMs, as in launch_advance: one warp per block for
+    // a pool that is not reordered (2e4 particles, 400 steps forward and back: 6.32 -> 6.04 ms), 64
+    // threads for a reordered one (2e5 particles x 1024 steps 39.8 -> 38.9 ms).
+    const unsigned long long warps = (a.n_particles + 31) / 32, given = (unsigned long long)blocks * 8;
+    const int nt = a.order ? 64 : 32;
+    const unsigned nb = (unsigned)(a.order ? given / 2 : (warps < given ? warps : given));
+    return cudaLaunchKernel(adj_fn(kind, a.g.dtype, a.g.pair, opt), dim3(nb), dim3(nt), args, 0, s);
 }
 
 cudaError_t launch_adjoint_forward(const AdvanceArgs& a, const AdjK& k, int blocks, cudaStream_t s)
