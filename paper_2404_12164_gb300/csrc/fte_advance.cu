@@ -28,12 +28,13 @@ static const void* single_fn(int kperp, int dtype)
     return single_dt<FTE_F32, MODE, LAY, shape>(kperp);
 }
 
-// the builds of block AMR (global tally, no cross-field diffusion): 16-bit records 3 blocks of
-// 256 threads per SM (at most 85 registers), FP32 records 4 blocks of 128 (128 registers, 16
-// warps).  With the options fixed and the shorter step the 16-warp build overtook the 20 warps
-// at 102 registers that FP32 ran before (1e7 particles x 320 steps: 145 ms with 20 warps and 160
-// bytes of spills, 136 with 16; 12 warps at 168 registers 157; 153 before).
-constexpr int kDenseBlocks = 768 / kThreads;
+// the builds of block AMR (global tally, no cross-field diffusion), 128 registers and 16 warps per
+// SM: FP32 records 4 blocks of 128 threads, 16-bit records 2 blocks of 256.  With the options
+// fixed and the shorter step 16 warps overtook the register-limited builds that ran before (FP32,
+// 1e7 particles x 320 steps: 145 ms with 20 warps at 102 registers, 136 with 16, 157 with 12 at
+// 168; BF16, 24 warps at 85 registers and 250 bytes of spills against 16: 3e6 particles x 192
+// steps 25.0 and 25.1 ms, 1e5 particles 1.40 and 1.30 ms).
+constexpr int kDenseBlocks = 512 / kThreads;
 constexpr int kAmr32Threads = 128;
 constexpr int kAmr32Blocks = 4;
 template <int LAY, int OPT = kOptAny, int SHAPE = kShapeLoop>

@@ -164,7 +164,7 @@ cudaError_t advance_occupancy(int kperp, int dtype, int mode, int nt, int pair, 
 int advance_opt(const GridK& g, const ParamsK& prm, int kperp, int mode);
 // Builds of the single-set step kernel: uniform grids 256 threads, two blocks per SM; block AMR
 // with the global tally and no cross-field diffusion FP32 records 4 blocks of 128 threads, 16-bit
-// records 3 blocks of 256 (see fte_advance.cu for the measurements).
+// records 2 blocks of 256 (see fte_advance.cu for the measurements).
 // advance_threads: threads per block of the build that advance_fn selects.
 int advance_threads(int kperp, int dtype, int mode, int amr);
 // the ensemble variants live in their own translation unit (fte_batched.cu)

@@ -340,9 +340,8 @@ __device__ __forceinline__ int set_of(const unsigned long long* end, int n_sets,
 // L1 keeps its whole capacity for the gather); kModeShared: an ensemble
 // (per-set parameters and tallies, the tallies of all sets in shared memory);
 // kModeGlobal: an ensemble with warp-merged FP64 atomics to the tally.
-// LAY: record layout (cell or pair), compile-time.  MINB: blocks per SM the single-set
-// kernel is compiled for (0: the register count ptxas chooses; 3: at most 85
-// registers, 24 warps per SM, for the longer dependent-load chains of block AMR).
+// LAY: record layout (cell or pair), compile-time.  MINB: blocks of NT threads per SM the
+// single-set kernel is compiled for (0: the register count the compiler chooses).
 // OPT: options fixed at compile time (kOptAny: none).
 template <bool KPERP, int DT, int MODE, int NT, int LAY, int MINB = 0, int OPT = kOptAny, int SHAPE = kShapeLoop>
 __global__ void __launch_bounds__(NT, single_set(MODE) ? MINB : 512 / NT) advance_kernel(const AdvanceArgs a, const BatchArgs b)
