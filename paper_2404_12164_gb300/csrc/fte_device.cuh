@@ -68,7 +68,7 @@ struct ObsK {
     float phi_scale;               // ring: longitude bin = floor(phi * nt / (2 pi))
 };
 
-// Per-step entry of the time table (built in FP64 by step_table_kernel).
+// Per-step entry of the time table (built in FP64 by setup_kernel).
 struct StepEntry {
     int s0, s1;              // bracketing snapshots
     float wt;                // weight of s1
