@@ -243,9 +243,11 @@ typedef struct fte_params {
                                   only: results do not depend on it); 0: no reordering */
     int32_t tally_layout;      /* fte_advance: FTE_LAYOUT_GLOBAL (or 0): lanes of a warp in the
                                   same bin are merged and added to the tally with FP64 atomics;
-                                  FTE_LAYOUT_SHARED: per-block histograms in shared memory
-                                  (at most 16384 bins), reduced after each launch.  The
-                                  counts are the same; the sums differ in rounding only */
+                                  FTE_LAYOUT_SHARED: the steps are counted per block in shared
+                                  memory (at most 16384 bins) and the counts reduced after each
+                                  launch; the sums go to the tally with FP64 atomics.  The
+                                  counts are the same; the sums differ in the order of the
+                                  FP64 additions only, as those of any two runs do */
 } fte_params;
 
 /* ---------------------------------------------------------------------------
@@ -402,12 +404,12 @@ fte_status fte_stream_load(const fte_background* bg, const void* host_snapshots,
    that must not call cudaMalloc once running).  Same arguments and stream
    semantics as fte_advance, but without the workspace: the scratch is a 24 MiB
    array that the library places in device memory statically, held by every GPU
-   that loads the library until the process exits.  It always tallies through
-   per-block shared-memory histograms (prm->tally_layout must still be a valid
+   that loads the library until the process exits.  It always counts the tallied
+   steps per block in shared memory (prm->tally_layout must still be a valid
    value and is otherwise not used) and never reorders the particles
    (prm->sort_every is not used): particle states, ledger and tally counts equal
    those of fte_advance with tally_layout = FTE_LAYOUT_SHARED, tally sums up to
-   the order of FP32 partial sums.  The first call on a device (with that device
+   the order of FP64 additions.  The first call on a device (with that device
    current) looks up the array's device address; make that first call before
    any stream capture.  That address belongs to the device's primary context: a
    cudaDeviceReset (or any teardown of that context) invalidates it, after which
@@ -443,9 +445,10 @@ typedef struct fte_launch_config {
     int32_t threads;           /* threads per block: 128 or 256 */
     int32_t steps_per_launch;  /* 1 .. 1024 steps per step-kernel launch; with prm->sort_every > 0
                                   the alive particles are reordered before every launch */
-    int32_t tally_layout;      /* FTE_LAYOUT_SHARED: every block keeps all sets' bins in shared
+    int32_t tally_layout;      /* FTE_LAYOUT_SHARED: every block counts all sets' steps in shared
                                   memory (n_sets * bins <= 16384 and the block must fit on an SM),
-                                  reduced into t after each launch; FTE_LAYOUT_GLOBAL: lanes of a
+                                  the counts reduced into t after each launch, the sums added to t
+                                  with FP64 atomics; FTE_LAYOUT_GLOBAL: lanes of a
                                   warp in the same bin are merged and added to t with FP64 atomics */
     int32_t pad;
 } fte_launch_config;

@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(256, 2) adj_forward_kernel(const AdvanceArgs a
         for (; s < a.n_end; ++s) {
             J += (double)(w * a.prm.dt * smooth_k(k, r, p, time_arg(k, s), nullptr, nullptr));
             st = step<false, DT, kModeNoTally, LAY, OPT, kAdjShape>(a, a.prm, I, 0, s, pid, x, y, z, mu, p, r, w,
-                                                                    nullptr, nullptr, nullptr, sc, noor, nrun);
+                                                                    nullptr, sc, noor, nrun);
             if (st != FTE_ALIVE) { ++s; break; }
         }
         // steps taken since the start of the run (a.n_table0), counting the one that ended it
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(256, 2) adj_replay_kernel(const AdvanceArgs a,
             sp[0] = x; sp[n] = y; sp[2 * n] = z; sp[3 * n] = mu; sp[4 * n] = p;
             if (s + 1 < e)
                 step<false, DT, kModeNoTally, LAY, OPT, kAdjShape>(a, a.prm, I, 0, s, pid, x, y, z, mu, p, r, w,
-                                                                   nullptr, nullptr, nullptr, sc, noor, nrun);
+                                                                   nullptr, sc, noor, nrun);
         }
         if (ce < e) {      // the start of the next chunk
             float* cp = k.carry + i;

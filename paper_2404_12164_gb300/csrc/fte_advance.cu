@@ -1,5 +1,5 @@
 // Transport kernels: the per-particle step loop with the fused occupancy tally,
-// the FP64 reduction of per-block partial histograms, the FP64 per-step time
+// the reduction of the blocks' step counts, the FP64 per-step time
 // table, the D_mumu normalisation integral and the intensity output.
 #include "fte_step.cuh"
 
@@ -282,43 +282,28 @@ cudaError_t launch_quantize(const float* f32, long long nrec, int row, int dtype
 }
 
 // ---------------------------------------------------------------------------
-// FP64 sum of the per-block partial histograms into the tally (deterministic
-// order: each bin's blocks are summed by 8 warps, then combined in order).
+// Sum of the blocks' step counts into the tally: each bin's blocks are summed by 8 warps.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) reduce_kernel(const float* __restrict__ part, int nblk,
-                                                     int nbins, double* S, double* S2,
+__global__ void __launch_bounds__(256) reduce_kernel(const unsigned* __restrict__ part, int nblk, int nbins,
                                                      unsigned long long* C)
 {
-    __shared__ double rs[8][32], rs2[8][32];
     __shared__ unsigned long long rc[8][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int b = blockIdx.x * 32 + lane;
-    double s = 0.0, s2 = 0.0;
     unsigned long long c = 0;
-    if (b < nbins) {
-        for (int k = wid; k < nblk; k += 8) {
-            const float* q = part + (size_t)k * 3 * nbins;
-            s += (double)q[b];
-            s2 += (double)q[nbins + b];
-            c += __float_as_uint(q[2 * nbins + b]);
-        }
-    }
-    rs[wid][lane] = s;
-    rs2[wid][lane] = s2;
+    if (b < nbins)
+        for (int k = wid; k < nblk; k += 8) c += part[(size_t)k * nbins + b];
     rc[wid][lane] = c;
     __syncthreads();
     if (wid == 0 && b < nbins) {
-        for (int k = 1; k < 8; ++k) { s += rs[k][lane]; s2 += rs2[k][lane]; c += rc[k][lane]; }
-        S[b] += s;
-        S2[b] += s2;
+        for (int k = 1; k < 8; ++k) c += rc[k][lane];
         C[b] += c;
     }
 }
 
-cudaError_t launch_reduce(const float* part, int nblk, int nbins, double* S, double* S2,
-                          unsigned long long* C, cudaStream_t s)
+cudaError_t launch_reduce(const unsigned* part, int nblk, int nbins, unsigned long long* C, cudaStream_t s)
 {
-    reduce_kernel<<<(nbins + 31) / 32, 256, 0, s>>>(part, nblk, nbins, S, S2, C);
+    reduce_kernel<<<(nbins + 31) / 32, 256, 0, s>>>(part, nblk, nbins, C);
     return cudaGetLastError();
 }
 

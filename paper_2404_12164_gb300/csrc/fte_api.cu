@@ -220,7 +220,7 @@ struct WsLayout {
     int threads;      // threads per block of its build (advance_threads)
 };
 
-constexpr int kMaxSmemBins = 16384;    // 3 x 4 B per bin in shared memory
+constexpr int kMaxSmemBins = 16384;    // bins that the shared-memory layout takes (4 B each)
 constexpr long long kChunkSteps = 1024;
 constexpr size_t kStreamGroupRuns = 8;   // snapshot intervals per fte_advance call of a streamed run
 // Work counters of the step kernel: one per SM range (warp_fetch_sm), for up to 1024 SM ids.
@@ -239,10 +239,10 @@ int device_sms(int device)
     return cache[device];
 }
 
-// shared memory of a single-set step kernel: the partial histogram, or none
+// shared memory of a single-set step kernel: the block's step counts, or none
 size_t single_smem(int mode, size_t nbins)
 {
-    return mode == kModeSingle ? 3 * sizeof(float) * (nbins ? nbins : 1) : 0;
+    return mode == kModeSingle ? sizeof(unsigned) * (nbins ? nbins : 1) : 0;
 }
 
 // Reordering scratch of fte_advance: one sort of the whole pool, or, when the pool is
@@ -330,7 +330,7 @@ fte_status layout(int device, int kperp, int dtype, int pair, int amr, int mode,
     L->off_table = off; off += (size_t)(n_steps > 0 ? n_steps : 1) * sizeof(StepEntry);
     off = (off + 255) & ~(size_t)255;
     L->off_part = off;
-    if (mode == kModeSingle) off += (size_t)L->blocks * 3 * (nbins ? nbins : 1) * sizeof(float);
+    if (mode == kModeSingle) off += (size_t)L->blocks * (nbins ? nbins : 1) * sizeof(unsigned);
     off = (off + 255) & ~(size_t)255;
     L->off_sort = off; off += sort_bytes;
     L->total = off;
@@ -653,7 +653,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
     a.n_table0 = n_start;
     a.table = ta.tab;
     a.norm = norm;
-    a.part = (float*)(w + L.off_part);
+    a.part = (unsigned*)(w + L.off_part);
     a.gS = t->S; a.gS2 = t->S2; a.gC = t->C;
     a.fetch = (unsigned long long*)(w + L.off_fetch);
     // per-SM ranges for FP32 records (L1 hits 95 -> 97 %; 16-bit records measured 2-3 % slower)
@@ -731,7 +731,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
         FTE_CUDA(launch_advance_timed(a, kperp, mode, blocks, smem, st, cap != cudaStreamCaptureStatusNone),
                  "step kernel launch");
         if (nb && mode == kModeSingle)
-            FTE_CUDA(launch_reduce(a.part, blocks, (int)nb, t->S, t->S2, t->C, st), "reduce launch");
+            FTE_CUDA(launch_reduce(a.part, blocks, (int)nb, t->C, st), "reduce launch");
     }
     return FTE_OK;
 }
@@ -965,13 +965,14 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
     if (n_end == n_start || P->count == 0) return FTE_OK;
 
     // scratch layout: fetch counter, normalisation, the time table of one
-    // launch, then per-block partial histograms
+    // launch, then the blocks' step counts
     const int kperp = prm->lambda_perp > 0.0 ? 1 : 0;
     // (the normalisation's partial sums are used up before the first table is written in their place)
     const size_t off_fetch = 0, off_norm = 64, off_table = 128 + 128 * sizeof(double), off_npart = off_table;
     static_assert(kNormPartials * sizeof(double) <= (size_t)kChunkSteps * sizeof(StepEntry), "norm scratch");
     const size_t off_part = (off_table + (size_t)kChunkSteps * sizeof(StepEntry) + 255) & ~(size_t)255;
-    const size_t part_block = 3 * sizeof(float) * (nb ? nb : 1);
+    // (12 bytes per bin set the largest tally that the call takes; the counts fill 4 of them)
+    const size_t part_block = 12 * (nb ? nb : 1);
     const int sms = device_sms(device);
     if (sms <= 0) return fail(FTE_ECUDA, "cannot query device %d", device);
     const size_t fit = (kNoAllocBytes - off_part) / part_block;
@@ -979,7 +980,7 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
         return fail(FTE_ENOMEM, "a tally of %zu bins needs %zu bytes of scratch per block; the "
                     "allocation-free variant holds %zu bytes, less than one block per SM (%d)",
                     nb, part_block, kNoAllocBytes, sms);
-    const size_t smem = part_block;
+    const size_t smem = single_smem(kModeSingle, nb);
     int per_sm = 0;
     FTE_CUDA(advance_occupancy(kperp, bg->grid.dtype, kModeSingle, kThreads, bg->grid.layout == FTE_LAYOUT_PAIR,
                                 bg->grid.amr_levels > 0, kOptAny, smem, &per_sm), "occupancy");
@@ -1009,7 +1010,8 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
     a.n_particles = P->count;
     a.table = (const StepEntry*)(w + off_table);
     a.norm = norm;
-    a.part = (float*)(w + off_part);
+    a.part = (unsigned*)(w + off_part);
+    a.gS = t->S; a.gS2 = t->S2;
     a.fetch = (unsigned long long*)(w + off_fetch);
     a.ledger_w = t->ledger_w; a.ledger_n = t->ledger_n;
 
@@ -1040,7 +1042,7 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
         a.n_table0 = c0;
         FTE_CUDA(cudaMemsetAsync(a.fetch, 0, sizeof(unsigned long long), st), "fetch reset");
         FTE_CUDA(launch_advance(a, g_no_batch, kperp, kModeSingle, kThreads, (int)blocks, smem, st), "step kernel launch");
-        if (nb) FTE_CUDA(launch_reduce(a.part, (int)blocks, (int)nb, t->S, t->S2, t->C, st), "reduce launch");
+        if (nb) FTE_CUDA(launch_reduce(a.part, (int)blocks, (int)nb, t->C, st), "reduce launch");
     }
     return FTE_OK;
 }
@@ -1062,7 +1064,7 @@ bool shared_fits(int n_sets, size_t nb) { return nb > 0 && shared_bins(n_sets, n
 
 size_t ens_smem(int mode, int n_sets, size_t nb)
 {
-    return mode == kModeShared ? 3 * sizeof(float) * shared_bins(n_sets, nb) : 0;
+    return mode == kModeShared ? sizeof(unsigned) * shared_bins(n_sets, nb) : 0;
 }
 
 fte_status ens_layout(int device, int kperp, int dtype, int pair, int mode, int opt, int nt, int n_sets, size_t nb,
@@ -1086,7 +1088,7 @@ fte_status ens_layout(int device, int kperp, int dtype, int pair, int mode, int 
     L->off_table = off; off += (size_t)(n_steps > 0 ? n_steps : 1) * sizeof(StepEntry);
     off = (off + 255) & ~(size_t)255;
     L->off_part = off;
-    if (mode == kModeShared) off += (size_t)L->blocks * 3 * shared_bins(n_sets, nb) * sizeof(float);
+    if (mode == kModeShared) off += (size_t)L->blocks * shared_bins(n_sets, nb) * sizeof(unsigned);
     off = (off + 255) & ~(size_t)255;
     L->off_sort = off; off += sort_bytes;
     L->total = off;
@@ -1199,7 +1201,7 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
     a.table = ta.tab;
     a.norm = norm;
     a.gS = t->S; a.gS2 = t->S2; a.gC = t->C;
-    a.part = (float*)(w + L.off_part);
+    a.part = (unsigned*)(w + L.off_part);
     a.fetch = (unsigned long long*)(w + L.off_fetch);
     // per-SM ranges for FP32 records (L1 hits 95 -> 97 %; 16-bit records measured 2-3 % slower)
     a.fetch_slots = bg->grid.dtype == FTE_F32 ? kFetchSlots : 0u;
@@ -1272,7 +1274,7 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
         else FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
         FTE_CUDA(launch_advance(a, b, kperp, cfg.mode, cfg.nt, blocks, smem, st), "step kernel launch");
         if (cfg.mode == kModeShared && nb)
-            FTE_CUDA(launch_reduce(a.part, blocks, reduce_bins, t->S, t->S2, t->C, st), "reduce launch");
+            FTE_CUDA(launch_reduce(a.part, blocks, reduce_bins, t->C, st), "reduce launch");
     }
     return FTE_OK;
 }

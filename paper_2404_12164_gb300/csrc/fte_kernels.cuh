@@ -47,7 +47,7 @@ struct AdvanceArgs {
     unsigned long long* gC;
     const uint32_t* order;        // alive particles in spatial order (NULL: all, by index)
     const unsigned* n_order;      // number of entries of `order` (device)
-    float* part;                  // per-block partial histograms [grid][3][nbins]
+    unsigned* part;               // shared modes: steps per bin of each block [grid][nbins]
     unsigned long long* fetch;    // particle counter for dynamic assignment
     unsigned fetch_slots;         // > 0: `fetch` holds that many per-SM range counters
     double* ledger_w;
@@ -171,8 +171,7 @@ int advance_threads(int kperp, int dtype, int mode, int amr);
 const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair, int opt);
 cudaError_t launch_advance_batched(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt,
                                    int blocks, size_t smem, cudaStream_t s);
-cudaError_t launch_reduce(const float* part, int nblk, int nbins, double* S, double* S2,
-                          unsigned long long* C, cudaStream_t s);
+cudaError_t launch_reduce(const unsigned* part, int nblk, int nbins, unsigned long long* C, cudaStream_t s);
 cudaError_t launch_step_table(const StepTableArgs& a, cudaStream_t s);
 // normalisation integral and step table (ta may be NULL); `part` holds kNormPartials doubles of scratch
 constexpr int kNormPartials = 272;

@@ -13,9 +13,12 @@ namespace fte {
 // leaves the launch: the steps tallied at one time are concentrated in a few bins
 // (one time bin, a few energy bins), so adding every step there would have tens of
 // thousands of threads contend for a handful of addresses.  The accumulators are
-// the FP64 tally in global memory (global modes) or the block's shared-memory
-// histogram (shared modes); the class-resolved tally (batch means) gains the same
-// sum in the particle's id class.
+// the FP64 tally in global memory; the shared modes count the steps in the block's
+// shared-memory histogram.  The sums go to FP64 in those too: FP32 partial sums per
+// block round in another order in every run (which block takes a particle is decided
+// by an atomic counter), so S and S2 of two equal runs differed by 5e-9 and up to 2e-8
+// in a bin.  The class-resolved tally (batch means) gains the same sum in the
+// particle's id class.
 // ---------------------------------------------------------------------------
 struct TallyRun {
     int bin;          // bin of the run of tallied steps, -1 before the first
@@ -23,20 +26,14 @@ struct TallyRun {
 };
 
 template <int MODE>
-__device__ __forceinline__ void tally_flush(const AdvanceArgs& a, float* shS, float* shS2, unsigned* shC,
-                                           TallyRun& t, float wdt, uint32_t pid)
+__device__ __forceinline__ void tally_flush(const AdvanceArgs& a, unsigned* shC, TallyRun& t, float wdt, uint32_t pid)
 {
     if (t.cnt == 0) return;
     const double d = (double)wdt, c = (double)t.cnt;
-    if (global_tally(MODE)) {
-        atomicAdd(&a.gS[t.bin], d * c);
-        atomicAdd(&a.gS2[t.bin], d * d * c);
-        atomicAdd(&a.gC[t.bin], (unsigned long long)t.cnt);
-    } else {
-        atomicAdd(&shS[t.bin], (float)(d * c));
-        atomicAdd(&shS2[t.bin], (float)(d * d * c));
-        atomicAdd(&shC[t.bin], t.cnt);
-    }
+    atomicAdd(&a.gS[t.bin], d * c);
+    atomicAdd(&a.gS2[t.bin], d * d * c);
+    if (global_tally(MODE)) atomicAdd(&a.gC[t.bin], (unsigned long long)t.cnt);
+    else atomicAdd(&shC[t.bin], t.cnt);
     if (a.cls) atomicAdd(a.cls + ((size_t)t.bin * FTE_NCLASS + (pid % FTE_NCLASS)), d * c);
     t.cnt = 0;
 }
@@ -78,7 +75,7 @@ template <bool KPERP, int DT, int MODE, int LAY, int OPT = kOptAny, int SHAPE = 
 __device__ __forceinline__ int step(const AdvanceArgs& a, const ParamsK& prm, float I, int sbin,
                                     long long n, uint32_t pid,
                                     float& x, float& y, float& z, float& mu, float& p, float& r, float w,
-                                    float* shS, float* shS2, unsigned* shC, const float* sc,
+                                    unsigned* shC, const float* sc,
                                     unsigned long long& noor, TallyRun& run)
 {
     const StepEntry* ep = a.table + (n - a.n_table0);
@@ -216,7 +213,7 @@ __device__ __forceinline__ int step(const AdvanceArgs& a, const ParamsK& prm, fl
             }
             if (bin >= 0) {
                 if (bin != run.bin) {
-                    tally_flush<MODE>(a, shS, shS2, shC, run, w * dt, pid);
+                    tally_flush<MODE>(a, shC, run, w * dt, pid);
                     run.bin = bin;
                 }
                 ++run.cnt;
@@ -335,10 +332,10 @@ __device__ __forceinline__ int set_of(const unsigned long long* end, int n_sets,
 
 // Persistent step kernel: each thread takes particles from a shared counter and
 // keeps each one in registers for all steps [n_start, n_end) of the launch.
-// MODE kModeSingle: one parameter set, tally in shared memory; kModeSingleGlobal:
+// MODE kModeSingle: one parameter set, tallied steps counted in shared memory; kModeSingleGlobal:
 // one parameter set, warp-merged FP64 atomics to the tally (no shared memory, so
 // L1 keeps its whole capacity for the gather); kModeShared: an ensemble
-// (per-set parameters and tallies, the tallies of all sets in shared memory);
+// (per-set parameters and tallies, the counts of all sets in shared memory);
 // kModeGlobal: an ensemble with warp-merged FP64 atomics to the tally.
 // LAY: record layout (cell or pair), compile-time.  MINB: blocks of NT threads per SM the
 // single-set kernel is compiled for (0: the register count the compiler chooses).
@@ -346,17 +343,14 @@ __device__ __forceinline__ int set_of(const unsigned long long* end, int n_sets,
 template <bool KPERP, int DT, int MODE, int NT, int LAY, int MINB = 0, int OPT = kOptAny, int SHAPE = kShapeLoop>
 __global__ void __launch_bounds__(NT, single_set(MODE) ? MINB : 512 / NT) advance_kernel(const AdvanceArgs a, const BatchArgs b)
 {
-    extern __shared__ float sh[];
+    extern __shared__ unsigned shC[];     // steps per bin
     const int nsh = global_tally(MODE) ? 0 : (MODE == kModeShared ? b.n_sets : 1) * a.nbins;
-    float* shS = sh;
-    float* shS2 = sh + nsh;
-    unsigned* shC = reinterpret_cast<unsigned*>(sh + 2 * nsh);
     __shared__ float sc[FTE_NFIELD];      // per-field scales of 16-bit storage
     constexpr int kSets = single_set(MODE) ? 1 : FTE_MAX_SETS;
     __shared__ unsigned long long s_end[kSets];
     __shared__ SetK s_set[kSets];
     __shared__ float s_I[kSets];
-    for (int q = threadIdx.x; q < 3 * nsh; q += NT) sh[q] = 0.f;
+    for (int q = threadIdx.x; q < nsh; q += NT) shC[q] = 0u;
     if (DT != FTE_F32 && threadIdx.x < FTE_NFIELD) sc[threadIdx.x] = __ldg(a.g.scale + threadIdx.x);
     if (!single_set(MODE)) {
         for (int s = threadIdx.x; s < b.n_sets; s += NT) {
@@ -403,8 +397,8 @@ __global__ void __launch_bounds__(NT, single_set(MODE) ? MINB : 512 / NT) advanc
         if (single_set(MODE)) {
             for (long long n = a.n_start; n < a.n_end; ++n) {
                 ++nsteps;
-                st = step<KPERP, DT, MODE, LAY, OPT, SHAPE>(a, a.prm, I0, 0, n, pid, x, y, z, mu, p, r, w, shS, shS2, shC, sc,
-                                                     noor, run);
+                st = step<KPERP, DT, MODE, LAY, OPT, SHAPE>(a, a.prm, I0, 0, n, pid, x, y, z, mu, p, r, w, shC, sc, noor,
+                                                     run);
                 if (st != FTE_ALIVE) break;
             }
         } else {
@@ -421,12 +415,12 @@ __global__ void __launch_bounds__(NT, single_set(MODE) ? MINB : 512 / NT) advanc
             const int sbin = s * a.nbins;
             for (long long n = a.n_start; n < a.n_end; ++n) {
                 ++nsteps;
-                st = step<KPERP, DT, MODE, LAY, OPT, SHAPE>(a, prm, I, sbin, n, pid, x, y, z, mu, p, r, w, shS, shS2, shC, sc,
-                                                     noor, run);
+                st = step<KPERP, DT, MODE, LAY, OPT, SHAPE>(a, prm, I, sbin, n, pid, x, y, z, mu, p, r, w, shC, sc, noor,
+                                                     run);
                 if (st != FTE_ALIVE) break;
             }
         }
-        tally_flush<MODE>(a, shS, shS2, shC, run, w * a.prm.dt, pid);
+        tally_flush<MODE>(a, shC, run, w * a.prm.dt, pid);
         a.x[i] = x; a.y[i] = y; a.z[i] = z; a.mu[i] = mu; a.p[i] = p;
         if (st != FTE_ALIVE) {
             a.status[i] = (uint8_t)st;
@@ -435,10 +429,10 @@ __global__ void __launch_bounds__(NT, single_set(MODE) ? MINB : 512 / NT) advanc
         }
     }
 
-    __syncthreads();   // all tally updates of this block are in shared memory
+    __syncthreads();   // all counts of this block are in shared memory
     if (!global_tally(MODE)) {
-        float* out = a.part + (size_t)blockIdx.x * 3 * nsh;
-        for (int q = threadIdx.x; q < 3 * nsh; q += NT) out[q] = sh[q];
+        unsigned* out = a.part + (size_t)blockIdx.x * nsh;
+        for (int q = threadIdx.x; q < nsh; q += NT) out[q] = shC[q];
     }
     nsteps = warp_sum_u64(nsteps);
     noor = warp_sum_u64(noor);
