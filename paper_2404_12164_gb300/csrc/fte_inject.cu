@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(kInjThreads) inject_kernel(const InjectArgs<NS
             const int q = (int)lane / g, t = t0 + (int)lane % g;
             const bool works = q < u && t < a.max_tries;
             const unsigned owner = works ? s_own[wid][q] : lane;
+            __syncwarp();                         // read by every lane before the next round's stores
             const uint32_t opid = pid - lane + owner;     // ids are consecutive within the warp
             float tr = 0.f, tth = 0.f, tph = 0.f;
             bool hit = false;
