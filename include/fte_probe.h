@@ -36,6 +36,13 @@ fte_status fte_probe_sectors(const void* buf, size_t bytes, int threads, int loa
 fte_status fte_probe_gather_l1(const void* buf, size_t bytes, int threads, int records, int spread,
                                float* dev_out, void* stream);
 
+/* A round of position attempts of fte_inject's kernel (HOST only, no GPU work): a warp with
+   n_pending particles that have no accepted position after t0 attempts of max_tries evaluates
+   *made attempts of each, on *width lanes each.  EINVAL unless 1 <= n_pending <= 32 and
+   0 <= t0 < max_tries. */
+fte_status fte_probe_attempt_round(int32_t n_pending, int32_t t0, int32_t max_tries, int32_t* width,
+                                   int32_t* made);
+
 /* Step-kernel launch timing for roofline accounting.  capacity > 0: from now on,
    every step-kernel launch of fte_advance (up to `capacity` of them) is bracketed by
    two CUDA events recorded on the stream of that launch (not while that stream is

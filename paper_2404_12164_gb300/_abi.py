@@ -160,6 +160,7 @@ SIGNATURES = {
     "fte_probe_sectors": (C.c_int, [C.c_void_p, C.c_size_t, C.c_int, C.c_int, C.c_void_p, C.c_void_p]),
     "fte_probe_gather_l1": (C.c_int, [C.c_void_p, C.c_size_t, C.c_int, C.c_int, C.c_int, C.c_void_p,
                                       C.c_void_p]),
+    "fte_probe_attempt_round": (C.c_int, [C.c_int32, C.c_int32, C.c_int32, _P(C.c_int32), _P(C.c_int32)]),
     "fte_probe_step_timing": (C.c_int, [C.c_int]),
     "fte_probe_step_intervals": (C.c_int, [C.c_void_p, C.c_int, _P(C.c_int)]),
     "fte_last_error": (C.c_char_p, []),

@@ -824,6 +824,18 @@ fte_status fte_probe_gather_l1(const void* buf, size_t bytes, int threads, int r
     return FTE_OK;
 }
 
+fte_status fte_probe_attempt_round(int32_t n_pending, int32_t t0, int32_t max_tries, int32_t* width,
+                                   int32_t* made)
+{
+    if (!width || !made) return fail(FTE_EINVAL, "NULL pointer");
+    if (n_pending < 1 || n_pending > 32 || t0 < 0 || t0 >= max_tries)
+        return fail(FTE_EINVAL, "need 1 to 32 particles and 0 <= t0 < max_tries");
+    const AttemptRound r(n_pending, t0, max_tries);
+    *width = r.width;
+    *made = r.made;
+    return FTE_OK;
+}
+
 fte_status fte_probe_step_timing(int capacity)
 {
     if (capacity < 0 || capacity > (1 << 20)) return fail(FTE_EINVAL, "capacity must be in [0, 2^20]");

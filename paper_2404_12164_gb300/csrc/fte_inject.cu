@@ -119,32 +119,31 @@ __global__ void __launch_bounds__(kInjThreads) inject_kernel(const InjectArgs<NS
         unsigned pend = __ballot_sync(0xffffffffu, mine);
         while (pend != 0u && t0 < a.max_tries) {
             const int u = __popc(pend);
-            int g = 1;                            // attempts per pending particle in this round
-            while (2 * g * u <= 32) g *= 2;
+            const AttemptRound round(u, t0, a.max_tries);
+            const int g = round.width;
             const bool waits = (pend >> lane) & 1u;
             const int rank = __popc(pend & ((1u << lane) - 1u));
             if (waits) s_own[wid][rank] = (unsigned char)lane;
             __syncwarp();
-            const int q = (int)lane / g, t = t0 + (int)lane % g;
-            const bool works = q < u && t < a.max_tries;
+            const int q = (int)lane / g, j = (int)lane % g;
+            const bool works = q < u && j < round.made;
             const unsigned owner = works ? s_own[wid][q] : lane;
             __syncwarp();                         // read by every lane before the next round's stores
             const uint32_t opid = pid - lane + owner;     // ids are consecutive within the warp
             float tr = 0.f, tth = 0.f, tph = 0.f;
             bool hit = false;
-            if (works) hit = attempt(k.g, a, c1, c2, t, opid, key, tr, tth, tph);
+            if (works) hit = attempt(k.g, a, c1, c2, t0 + j, opid, key, tr, tth, tph);
             const unsigned hits = __ballot_sync(0xffffffffu, hit);
             const unsigned seg = waits ? (hits >> (rank * g)) & (g == 32 ? 0xffffffffu : (1u << g) - 1u) : 0u;
             // the accepted attempt, or the last one of a particle that runs out of attempts
-            const int last = min(g, a.max_tries - t0) - 1;
-            const int src = waits ? rank * g + (seg ? __ffs(seg) - 1 : last) : (int)lane;
+            const int src = waits ? rank * g + (seg ? __ffs(seg) - 1 : round.made - 1) : (int)lane;
             const float fr = __shfl_sync(0xffffffffu, tr, src);
             const float fth = __shfl_sync(0xffffffffu, tth, src);
             const float fph = __shfl_sync(0xffffffffu, tph, src);
             if (waits) { r = fr; th = fth; ph = fph; }
             if (seg) ok = true;
             pend = __ballot_sync(0xffffffffu, waits && !seg);
-            t0 += g;
+            t0 += round.made;
         }
     }
     double wsum = 0.0;

@@ -103,6 +103,19 @@ struct InjectSet {
     unsigned long long offset, n; // pool entries [offset, offset + n)
 };
 
+// One round of shared position attempts (inject_kernel) after t0 < max_tries attempts of each of
+// the warp's n_pending (1 .. 32) particles that have none accepted yet: `width` consecutive
+// attempts of each, particle q on lanes q width .. q width + width - 1, of which `made` are within
+// the limit.  No sum goes beyond max_tries, which may be the largest int.
+struct AttemptRound {
+    int width, made;
+    __host__ __device__ __forceinline__ AttemptRound(int n_pending, int t0, int max_tries) : width(1)
+    {
+        while (2 * width * n_pending <= 32) width *= 2;
+        made = max_tries - t0 < width ? max_tries - t0 : width;
+    }
+};
+
 // NS injections in one launch: NS = 1, or up to FTE_MAX_SETS of an ensemble.
 template <int NS>
 struct InjectArgs {
