@@ -384,6 +384,34 @@ InjectSet inject_set(const fte_inject_spec* spec, uint64_t offset, uint64_t n)
     return a;
 }
 
+// Whether one kernel may clear these arrays.  A memset finds the memory by its address and takes
+// any alignment; a kernel runs on the current device and writes 8-byte words.  So every array has
+// to be aligned device memory of the current device and the stream one of that device; while it is
+// being captured, the memsets go into the graph (the look-ups are no calls for a capture, this
+// stream's or, hence the mode, another's).  Six look-ups and one launch against six memsets: 2000
+// particles x 200 steps 369 us and 385 us.
+bool zero_in_one_launch(const ZeroArgs& z, cudaStream_t st)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+    int cur = 0, dev = 0;
+    bool ok = cudaGetDevice(&cur) == cudaSuccess && cudaStreamGetDevice(st, &dev) == cudaSuccess && dev == cur;
+    for (int k = 0; k < 6 && ok; ++k) {
+        if (!z.n[k]) continue;
+        cudaPointerAttributes at;
+        ok = (uintptr_t)z.p[k] % 8 == 0 && cudaPointerGetAttributes(&at, z.p[k]) == cudaSuccess &&
+             at.type == cudaMemoryTypeDevice && at.device == cur;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!ok) cudaGetLastError();       // a refused look-up is no error of the call
+    return ok;
+}
+
 template <int NS>
 void inject_pool(const fte_particles* P, const fte_background* bg, const fte_tally_buf* t, InjectArgs<NS>* a)
 {
@@ -510,7 +538,12 @@ fte_status fte_tally_reset(const fte_tally_buf* t, void* stream)
     if (t->S_class && nb) set(3, t->S_class, nb * FTE_NCLASS);
     set(4, t->ledger_w, FTE_LEDGER);
     set(5, t->ledger_n, FTE_LEDGER);
-    FTE_CUDA(launch_zero(z, st), "tally reset");
+    if (zero_in_one_launch(z, st)) {
+        FTE_CUDA(launch_zero(z, st), "tally reset");
+        return FTE_OK;
+    }
+    for (int k = 0; k < 6; ++k)
+        if (z.n[k]) FTE_CUDA(cudaMemsetAsync(z.p[k], 0, z.n[k] * 8, st), "tally reset");
     return FTE_OK;
 }
 
