@@ -606,7 +606,10 @@ static const void* adj_fn_dtype(int kind, int dtype)
     return adj_kernel<FTE_F32, LAY, OPT>(kind);
 }
 
-int adjoint_opt(const GridK& g, const ParamsK& prm) { return advance_opt(g, prm, 0, kModeSingleGlobal); }
+int adjoint_opt(const GridK& g, const ParamsK& prm)
+{
+    return advance_opt(g, prm, 0, kModeSingleGlobal, true, 0, 0);
+}
 
 // record layout and, for the common options (advance_opt: cell records only), the options fixed
 // at compile time, as for the step kernels

@@ -47,6 +47,13 @@ static const void* dense_fn(int dtype)
     return (const void*)advance_kernel<false, FTE_F32, kModeSingleGlobal, kAmr32Threads, LAY, kAmr32Blocks, OPT, SHAPE>;
 }
 
+// FP32 records, 5 blocks of 128 threads, 20 warps per SM at 102 registers (see advance_opt)
+template <int LAY>
+static const void* warps_fn()
+{
+    return (const void*)advance_kernel<false, FTE_F32, kModeSingleGlobal, kAmr32Threads, LAY, 5>;
+}
+
 // near: the build with the reach test of the observers (kShapeNear)
 template <int DT>
 static const void* linear_dt(bool near)
@@ -70,8 +77,16 @@ static bool dense_variant(int kperp, int mode, int amr)
     return mode == kModeSingleGlobal && !kperp && amr;
 }
 
-int advance_opt(const GridK& g, const ParamsK& prm, int kperp, int mode)
+int advance_opt(const GridK& g, const ParamsK& prm, int kperp, int mode, bool ordered, unsigned long long n, int sms)
 {
+    // FP32 block AMR with linear r, not reordered, more than 8 warps of particles per SM: the general
+    // kernel in the build of 20 warps per SM.  Its 16-warp build, the faster one everywhere else, falls
+    // behind there (per launch of 192 - 384 steps, 16 against 20 warps: 1e6 particles 37.2 and 32.2 ms,
+    // in pair records 41.4 and 28.4; 3e5 15.4 and 12.9; 1.2e5 9.9 and 8.1; 6e4 5.3 and 4.3; but 2e4
+    // 2.9 and 3.9; reordered, 1.2e5: 3.0 and 3.6).  Logarithmic r and 16-bit records do not show it.
+    if (mode == kModeSingleGlobal && !kperp && g.amr > 0 && !g.radial && g.dtype == FTE_F32 && !ordered &&
+        n > (unsigned long long)sms * 256)
+        return kOptAnyWarps;
     const bool common = prm.dmumu == 0 && !prm.use_rig && prm.p_update == 0 && prm.dvdt_term;
     if (!common || kperp || g.pair || !global_tally(mode)) return kOptAny;
     if (g.amr > 0) return g.radial && mode == kModeSingleGlobal ? kOptAmrLog : kOptAny;
@@ -90,6 +105,7 @@ static const void* advance_fn(int kperp, int dtype, int mode, int nt, int pair, 
 {
     if (!single_set(mode)) return advance_fn_batched(kperp, dtype, mode, nt, pair, opt);
     if (nt != advance_threads(kperp, dtype, mode, amr)) return nullptr;
+    if (opt == kOptAnyWarps) return pair ? warps_fn<kLayPair>() : warps_fn<kLayCell>();
     if (opt == kOptAmrLog) return dense_fn<kLayCell, kOptAmrLog, kShapeNear>(dtype);
     if (opt == kOptLinear) return linear_fn(dtype, near);
     if (dense_variant(kperp, mode, amr)) return pair ? dense_fn<kLayPair>(dtype) : dense_fn<kLayCell>(dtype);
@@ -109,14 +125,13 @@ cudaError_t advance_occupancy(int kperp, int dtype, int mode, int nt, int pair, 
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, nt, smem);
 }
 
-cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt, int blocks,
+cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt, int opt, int blocks,
                            size_t smem, cudaStream_t s)
 {
-    if (!single_set(mode)) return launch_advance_batched(a, b, kperp, mode, nt, blocks, smem, s);
+    if (!single_set(mode)) return launch_advance_batched(a, b, kperp, mode, nt, opt, blocks, smem, s);
     // reordered, or at most one particle per thread (see kShapeNear)
     const bool near = a.order || a.n_particles <= (unsigned long long)blocks * nt;
-    const void* fn = advance_fn(kperp, a.g.dtype, mode, nt, a.g.pair, a.g.amr > 0, advance_opt(a.g, a.prm, kperp, mode),
-                                near);
+    const void* fn = advance_fn(kperp, a.g.dtype, mode, nt, a.g.pair, a.g.amr > 0, opt, near);
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {(void*)&a, (void*)&b};
     // The global-tally kernels share nothing within a block, so blocks only decide how warps

@@ -268,16 +268,16 @@ struct StepTiming {
 };
 StepTiming g_timing;
 
-cudaError_t launch_advance_timed(const AdvanceArgs& a, int kperp, int mode, int blocks, size_t smem, cudaStream_t s,
-                                 bool capturing)
+cudaError_t launch_advance_timed(const AdvanceArgs& a, int kperp, int mode, int opt, int blocks, size_t smem,
+                                 cudaStream_t s, bool capturing)
 {
     const int nt = advance_threads(kperp, a.g.dtype, mode, a.g.amr > 0);
     if (!g_timing.on.load(std::memory_order_relaxed) || capturing)
-        return launch_advance(a, g_no_batch, kperp, mode, nt, blocks, smem, s);
+        return launch_advance(a, g_no_batch, kperp, mode, nt, opt, blocks, smem, s);
     std::lock_guard<std::mutex> lock(g_timing.mu);
     const bool rec = g_timing.used + 2 <= (int)g_timing.ev.size();
     if (rec) cudaEventRecord(g_timing.ev[g_timing.used], s);
-    const cudaError_t e = launch_advance(a, g_no_batch, kperp, mode, nt, blocks, smem, s);
+    const cudaError_t e = launch_advance(a, g_no_batch, kperp, mode, nt, opt, blocks, smem, s);
     if (rec) {
         cudaEventRecord(g_timing.ev[g_timing.used + 1], s);
         g_timing.used += 2;
@@ -296,15 +296,15 @@ struct SideStream {
     }
 };
 
-// The compile-time options of the step kernel for these parameters (advance_opt).  The
-// workspace of the global-tally kernels does not depend on them.
-int params_opt(const GridK& g, const fte_params* prm, int kperp, int mode)
+// The step kernel's build for these parameters and a pool of n particles (advance_opt).  The
+// workspace of the global-tally kernels does not depend on it.
+int params_opt(const GridK& g, const fte_params* prm, int kperp, int mode, unsigned long long n, int device)
 {
     ParamsK k;
     memset(&k, 0, sizeof(k));
     k.dmumu = prm->dmumu; k.p_update = prm->p_update; k.dvdt_term = prm->dvdt_term;
     k.use_rig = (prm->p_ref > 0.0 && prm->alpha != 0.0) ? 1 : 0;
-    return advance_opt(g, k, kperp, mode);
+    return advance_opt(g, k, kperp, mode, prm->sort_every > 0, n, device_sms(device));
 }
 
 fte_status layout(int device, int kperp, int dtype, int pair, int amr, int mode, int opt, size_t nbins,
@@ -637,7 +637,8 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
     const GridK gk = make_gridk(bg);
     const int sorting = prm->sort_every > 0;
     WsLayout L;
-    s = layout(device, kperp, bg->grid.dtype, gk.pair, gk.amr > 0, mode, params_opt(gk, prm, kperp, mode), nb, nsteps,
+    const int opt = params_opt(gk, prm, kperp, mode, P->count, device);
+    s = layout(device, kperp, bg->grid.dtype, gk.pair, gk.amr > 0, mode, opt, nb, nsteps,
                sorting ? advance_sort_bytes(gk, P->count) : 0,
                &L);
     if (s != FTE_OK) return s;
@@ -706,7 +707,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
     const size_t smem = single_smem(mode, nb);
     int per_sm = 0;
     FTE_CUDA(advance_occupancy(kperp, bg->grid.dtype, mode, L.threads, bg->grid.layout == FTE_LAYOUT_PAIR, gk.amr > 0,
-                               params_opt(gk, prm, kperp, mode), smem, &per_sm), "occupancy");
+                               opt, smem, &per_sm), "occupancy");
 
     // Two halves on two streams: while the last particles of one half's launch run, the
     // other half's reordering and launch fill the idle SMs (the step kernel launches one
@@ -748,7 +749,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
                 ah[k].n_start = c0;
                 ah[k].n_end = (c0 + chunk < n_end) ? c0 + chunk : n_end;
                 FTE_CUDA(launch_sort(sh[k], c0 == n_start, ah[k].fetch, kFetchSlots, hs[k]), "sort launch");
-                FTE_CUDA(launch_advance_timed(ah[k], kperp, mode, blocks, smem, hs[k], false), "step kernel launch");
+                FTE_CUDA(launch_advance_timed(ah[k], kperp, mode, opt, blocks, smem, hs[k], false), "step kernel launch");
             }
         }
         FTE_CUDA(cudaEventRecord(side.join, side.s), "join");
@@ -761,7 +762,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
         a.n_end = (c0 + chunk < n_end) ? c0 + chunk : n_end;
         if (sorting) FTE_CUDA(launch_sort(sa, c0 == n_start, a.fetch, kFetchSlots, st), "sort launch");
         else FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
-        FTE_CUDA(launch_advance_timed(a, kperp, mode, blocks, smem, st, cap != cudaStreamCaptureStatusNone),
+        FTE_CUDA(launch_advance_timed(a, kperp, mode, opt, blocks, smem, st, cap != cudaStreamCaptureStatusNone),
                  "step kernel launch");
         if (nb && mode == kModeSingle)
             FTE_CUDA(launch_reduce(a.part, blocks, (int)nb, t->C, st), "reduce launch");
@@ -1086,7 +1087,7 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
         a.n_end = c1;
         a.n_table0 = c0;
         FTE_CUDA(cudaMemsetAsync(a.fetch, 0, sizeof(unsigned long long), st), "fetch reset");
-        FTE_CUDA(launch_advance(a, g_no_batch, kperp, kModeSingle, kThreads, (int)blocks, smem, st), "step kernel launch");
+        FTE_CUDA(launch_advance(a, g_no_batch, kperp, kModeSingle, kThreads, kOptAny, (int)blocks, smem, st), "step kernel launch");
         if (nb) FTE_CUDA(launch_reduce(a.part, (int)blocks, (int)nb, t->C, st), "reduce launch");
     }
     return FTE_OK;
@@ -1185,8 +1186,8 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
     const GridK gk = make_gridk(bg);
     const int sorting = prm->sort_every > 0;
     EnsLayout L;
-    fte_status s = ens_layout(device, kperp, bg->grid.dtype, gk.pair, cfg.mode, params_opt(gk, prm, kperp, cfg.mode),
-                              cfg.nt, n_sets, nb, nsteps,
+    const int opt = params_opt(gk, prm, kperp, cfg.mode, P->count, device);
+    fte_status s = ens_layout(device, kperp, bg->grid.dtype, gk.pair, cfg.mode, opt, cfg.nt, n_sets, nb, nsteps,
                               sorting ? advance_sort_bytes(gk, P->count) : 0, &L);
     if (s != FTE_OK) return s;
     if (ws_bytes < L.total) return fail(FTE_ENOMEM, "workspace has %zu bytes, needs %zu", ws_bytes, L.total);
@@ -1303,7 +1304,7 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
                 ah[k].n_start = c0;
                 ah[k].n_end = (c0 + cfg.steps < n_end) ? c0 + cfg.steps : n_end;
                 FTE_CUDA(launch_sort(sh[k], c0 == n_start, ah[k].fetch, kFetchSlots, hs[k]), "sort launch");
-                FTE_CUDA(launch_advance(ah[k], bh[k], kperp, cfg.mode, cfg.nt, blocks, smem, hs[k]),
+                FTE_CUDA(launch_advance(ah[k], bh[k], kperp, cfg.mode, cfg.nt, opt, blocks, smem, hs[k]),
                          "step kernel launch");
             }
         }
@@ -1317,7 +1318,7 @@ fte_status ens_run(fte_particles* P, const fte_background* bg, const fte_params*
         a.n_end = (c0 + cfg.steps < n_end) ? c0 + cfg.steps : n_end;
         if (sorting) FTE_CUDA(launch_sort(sa, c0 == n_start, a.fetch, kFetchSlots, st), "sort launch");
         else FTE_CUDA(cudaMemsetAsync(a.fetch, 0, kFetchBytes, st), "fetch reset");
-        FTE_CUDA(launch_advance(a, b, kperp, cfg.mode, cfg.nt, blocks, smem, st), "step kernel launch");
+        FTE_CUDA(launch_advance(a, b, kperp, cfg.mode, cfg.nt, opt, blocks, smem, st), "step kernel launch");
         if (cfg.mode == kModeShared && nb)
             FTE_CUDA(launch_reduce(a.part, blocks, reduce_bins, t->C, st), "reduce launch");
     }

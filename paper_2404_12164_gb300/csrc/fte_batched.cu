@@ -56,9 +56,9 @@ const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair,
 }
 
 cudaError_t launch_advance_batched(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt,
-                                   int blocks, size_t smem, cudaStream_t s)
+                                   int opt, int blocks, size_t smem, cudaStream_t s)
 {
-    const void* fn = advance_fn_batched(kperp, a.g.dtype, mode, nt, a.g.pair, advance_opt(a.g, a.prm, kperp, mode));
+    const void* fn = advance_fn_batched(kperp, a.g.dtype, mode, nt, a.g.pair, opt);
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {(void*)&a, (void*)&b};
     return cudaLaunchKernel(fn, dim3(blocks), dim3(nt), args, smem, s);

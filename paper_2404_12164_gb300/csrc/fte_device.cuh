@@ -129,6 +129,7 @@ __device__ __forceinline__ float energy_of(float p)
 // ms; 1e6 particles over 4 days 595 -> 577 ms together with the register limit (kMinBlocks).
 // ---------------------------------------------------------------------------
 constexpr int kOptAny = 0, kOptLinear = 1, kOptAmrLog = 2;
+constexpr int kOptAnyWarps = 3;    // launches only: the kernel of kOptAny in a build for more warps (advance_opt)
 
 template <int OPT>
 __device__ __forceinline__ bool opt_amr(const GridK& g) { return OPT == kOptAny ? g.amr > 0 : OPT == kOptAmrLog; }

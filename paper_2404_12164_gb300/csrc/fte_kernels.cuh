@@ -166,24 +166,24 @@ struct AdjK {
 // launchers (return cudaGetLastError())
 // step kernel of (kperp, dtype, mode, threads per block); for the single-set modes nt must
 // be advance_threads() of the same arguments
-cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt, int blocks,
+cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt, int opt, int blocks,
                            size_t smem, cudaStream_t s);
 // resident blocks per SM of a step kernel (`pair`: record layout of a single-set kernel)
 cudaError_t advance_occupancy(int kperp, int dtype, int mode, int nt, int pair, int amr, int opt, size_t smem,
                               int* blocks_per_sm);
-// the options (kOptAny, ...) that a launch with these parameters can have fixed at compile time:
-// global tally, cell records and no cross-field diffusion (the other builds take them all from
-// the parameters)
-int advance_opt(const GridK& g, const ParamsK& prm, int kperp, int mode);
+// the build (kOptAny, ...) for a pool of n particles with these parameters on a device with `sms`
+// SMs: the options fixed at compile time with the global tally, cell records and no cross-field
+// diffusion (the other builds take them all from the parameters)
+int advance_opt(const GridK& g, const ParamsK& prm, int kperp, int mode, bool ordered, unsigned long long n, int sms);
 // Builds of the single-set step kernel: uniform grids 256 threads, two blocks per SM; block AMR
-// with the global tally and no cross-field diffusion FP32 records 4 blocks of 128 threads, 16-bit
-// records 2 blocks of 256 (see fte_advance.cu for the measurements).
+// with the global tally and no cross-field diffusion FP32 records 4 blocks of 128 threads (5 for
+// kOptAnyWarps), 16-bit records 2 blocks of 256 (see fte_advance.cu for the measurements).
 // advance_threads: threads per block of the build that advance_fn selects.
 int advance_threads(int kperp, int dtype, int mode, int amr);
 // the ensemble variants live in their own translation unit (fte_batched.cu)
 const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair, int opt);
 cudaError_t launch_advance_batched(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt,
-                                   int blocks, size_t smem, cudaStream_t s);
+                                   int opt, int blocks, size_t smem, cudaStream_t s);
 cudaError_t launch_reduce(const unsigned* part, int nblk, int nbins, unsigned long long* C, cudaStream_t s);
 cudaError_t launch_step_table(const StepTableArgs& a, cudaStream_t s);
 // normalisation integral and step table (ta may be NULL); `part` holds kNormPartials doubles of scratch
