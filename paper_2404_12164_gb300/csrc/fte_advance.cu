@@ -103,10 +103,11 @@ int advance_threads(int kperp, int dtype, int mode, int amr)
 // in one with these fixed
 static const void* advance_fn(int kperp, int dtype, int mode, int nt, int pair, int amr, int opt, bool near = true)
 {
-    if (!single_set(mode)) return advance_fn_batched(kperp, dtype, mode, nt, pair, opt);
+    if (!single_set(mode)) return advance_fn_batched(kperp, dtype, mode, nt, pair, opt, near);
     if (nt != advance_threads(kperp, dtype, mode, amr)) return nullptr;
     if (opt == kOptAnyWarps) return pair ? warps_fn<kLayPair>() : warps_fn<kLayCell>();
-    if (opt == kOptAmrLog) return dense_fn<kLayCell, kOptAmrLog, kShapeNear>(dtype);
+    if (opt == kOptAmrLog)
+        return near ? dense_fn<kLayCell, kOptAmrLog, kShapeNear>(dtype) : dense_fn<kLayCell, kOptAmrLog>(dtype);
     if (opt == kOptLinear) return linear_fn(dtype, near);
     if (dense_variant(kperp, mode, amr)) return pair ? dense_fn<kLayPair>(dtype) : dense_fn<kLayCell>(dtype);
     if (mode == kModeSingleGlobal)
@@ -128,9 +129,9 @@ cudaError_t advance_occupancy(int kperp, int dtype, int mode, int nt, int pair, 
 cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt, int opt, int blocks,
                            size_t smem, cudaStream_t s)
 {
-    if (!single_set(mode)) return launch_advance_batched(a, b, kperp, mode, nt, opt, blocks, smem, s);
     // reordered, or at most one particle per thread (see kShapeNear)
     const bool near = a.order || a.n_particles <= (unsigned long long)blocks * nt;
+    if (!single_set(mode)) return launch_advance_batched(a, b, kperp, mode, nt, opt, near, blocks, smem, s);
     const void* fn = advance_fn(kperp, a.g.dtype, mode, nt, a.g.pair, a.g.amr > 0, opt, near);
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {(void*)&a, (void*)&b};

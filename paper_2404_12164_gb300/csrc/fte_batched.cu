@@ -26,25 +26,30 @@ static const void* pick_layout(int kperp, int dtype, int pair)
     return pair ? pick<MODE, NT, kLayPair>(kperp, dtype) : pick<MODE, NT, kLayCell>(kperp, dtype);
 }
 
-// global tally, cell records, no cross-field diffusion, options fixed (advance_opt)
+// global tally, cell records, no cross-field diffusion, options fixed (advance_opt); near: with
+// the reach test of the observers (kShapeNear)
 template <int DT, int NT>
-static const void* pick_linear_dt()
+static const void* pick_linear_dt(bool near)
 {
-    return (const void*)advance_kernel<false, DT, kModeGlobal, NT, kLayCell, 0, kOptLinear,
-                                       kShapeUnroll | kShapeNormals | kShapeNear>;
+    constexpr int shape = kShapeUnroll | kShapeNormals;
+    return near ? (const void*)advance_kernel<false, DT, kModeGlobal, NT, kLayCell, 0, kOptLinear, shape | kShapeNear>
+                : (const void*)advance_kernel<false, DT, kModeGlobal, NT, kLayCell, 0, kOptLinear, shape>;
 }
 
 template <int NT>
-static const void* pick_linear(int dtype)
+static const void* pick_linear(int dtype, bool near)
 {
-    if (dtype == FTE_BF16) return pick_linear_dt<FTE_BF16, NT>();
-    if (dtype == FTE_F16) return pick_linear_dt<FTE_F16, NT>();
-    return pick_linear_dt<FTE_F32, NT>();
+    if (dtype == FTE_BF16) return pick_linear_dt<FTE_BF16, NT>(near);
+    if (dtype == FTE_F16) return pick_linear_dt<FTE_F16, NT>(near);
+    return pick_linear_dt<FTE_F32, NT>(near);
 }
 
-const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair, int opt)
+const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair, int opt, bool near)
 {
-    if (opt == kOptLinear) return nt == 128 ? pick_linear<128>(dtype) : (nt == 256 ? pick_linear<256>(dtype) : nullptr);
+    if (opt == kOptLinear) {
+        if (nt == 128) return pick_linear<128>(dtype, near);
+        return nt == 256 ? pick_linear<256>(dtype, near) : nullptr;
+    }
     if (mode == kModeShared) {
         if (nt == 128) return pick_layout<kModeShared, 128>(kperp, dtype, pair);
         if (nt == 256) return pick_layout<kModeShared, 256>(kperp, dtype, pair);
@@ -56,9 +61,9 @@ const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair,
 }
 
 cudaError_t launch_advance_batched(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt,
-                                   int opt, int blocks, size_t smem, cudaStream_t s)
+                                   int opt, bool near, int blocks, size_t smem, cudaStream_t s)
 {
-    const void* fn = advance_fn_batched(kperp, a.g.dtype, mode, nt, a.g.pair, opt);
+    const void* fn = advance_fn_batched(kperp, a.g.dtype, mode, nt, a.g.pair, opt, near);
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {(void*)&a, (void*)&b};
     return cudaLaunchKernel(fn, dim3(blocks), dim3(nt), args, smem, s);

@@ -181,9 +181,9 @@ int advance_opt(const GridK& g, const ParamsK& prm, int kperp, int mode, bool or
 // advance_threads: threads per block of the build that advance_fn selects.
 int advance_threads(int kperp, int dtype, int mode, int amr);
 // the ensemble variants live in their own translation unit (fte_batched.cu)
-const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair, int opt);
+const void* advance_fn_batched(int kperp, int dtype, int mode, int nt, int pair, int opt, bool near);
 cudaError_t launch_advance_batched(const AdvanceArgs& a, const BatchArgs& b, int kperp, int mode, int nt,
-                                   int opt, int blocks, size_t smem, cudaStream_t s);
+                                   int opt, bool near, int blocks, size_t smem, cudaStream_t s);
 cudaError_t launch_reduce(const unsigned* part, int nblk, int nbins, unsigned long long* C, cudaStream_t s);
 cudaError_t launch_step_table(const StepTableArgs& a, cudaStream_t s);
 // normalisation integral and step table (ta may be NULL); `part` holds kNormPartials doubles of scratch
