@@ -20,8 +20,11 @@
 
 namespace fte {
 
-// the form of the forward and replay steps (adjoint passes of 2e5 particles 43.3 -> 42.6 ms)
-constexpr int kAdjShape = kShapeUnroll | kShapeNormals;
+// The form of the forward and replay steps: both snapshots' gathers in one block (adjoint passes of
+// 2e5 particles 43.3 -> 42.6 ms), but for pools of several waves on block AMR that are not reordered,
+// which lose 2.5 % by it (2e5 particles, 128 steps forward and back 15.7 and 15.3 ms; 5e3 on the
+// general kernel 2.17 and 2.23, reordered 2e5 7.0 and 7.2).
+constexpr int kAdjShape = kShapeUnroll | kShapeNormals, kAdjShapeScattered = kShapeNormals;
 
 // ---------------------------------------------------------------------------
 // d/dq and d/dH (quasi-linear) or d/deps (Eq. 5) of the normalisation integral,
@@ -395,7 +398,7 @@ __device__ void step_vjp(const AdvanceArgs& a, float I, float rq, float rh, long
 // in spatial order from a.order when reordering is on) stores its checkpoint,
 // runs the segment's steps and adds its observable to J_part.
 // ---------------------------------------------------------------------------
-template <int DT, int LAY, int OPT>
+template <int DT, int LAY, int OPT, int SHAPE>
 __global__ void __launch_bounds__(256, 2) adj_forward_kernel(const AdvanceArgs a, const AdjK k)
 {
     __shared__ float sc[FTE_NFIELD];
@@ -427,7 +430,7 @@ __global__ void __launch_bounds__(256, 2) adj_forward_kernel(const AdvanceArgs a
         float r = radius(x, y, z);
         for (; s < a.n_end; ++s) {
             J += (double)(w * a.prm.dt * smooth_k(k, r, p, time_arg(k, s), nullptr, nullptr));
-            st = step<false, DT, kModeNoTally, LAY, OPT, kAdjShape>(a, a.prm, I, 0, s, pid, x, y, z, mu, p, r, w,
+            st = step<false, DT, kModeNoTally, LAY, OPT, SHAPE>(a, a.prm, I, 0, s, pid, x, y, z, mu, p, r, w,
                                                                     nullptr, sc, noor, nrun);
             if (st != FTE_ALIVE) { ++s; break; }
         }
@@ -459,7 +462,7 @@ __global__ void __launch_bounds__(256, 2) adj_forward_kernel(const AdvanceArgs a
 // the stored states, carrying the adjoints between launches in k.adj.  The launch
 // of the run's first chunk adds the injection-index term and reduces the gradients.
 // ---------------------------------------------------------------------------
-template <int DT, int LAY, int OPT>
+template <int DT, int LAY, int OPT, int SHAPE>
 __global__ void __launch_bounds__(256, 2) adj_replay_kernel(const AdvanceArgs a, const AdjK k)
 {
     __shared__ float sc[FTE_NFIELD];
@@ -493,7 +496,7 @@ __global__ void __launch_bounds__(256, 2) adj_replay_kernel(const AdvanceArgs a,
             float* sp = k.scratch + (size_t)(s - n0) * 5 * n + f;
             sp[0] = x; sp[n] = y; sp[2 * n] = z; sp[3 * n] = mu; sp[4 * n] = p;
             if (s + 1 < e)
-                step<false, DT, kModeNoTally, LAY, OPT, kAdjShape>(a, a.prm, I, 0, s, pid, x, y, z, mu, p, r, w,
+                step<false, DT, kModeNoTally, LAY, OPT, SHAPE>(a, a.prm, I, 0, s, pid, x, y, z, mu, p, r, w,
                                                                    nullptr, sc, noor, nrun);
         }
         if (ce < e) {      // the start of the next chunk
@@ -590,20 +593,27 @@ __global__ void __launch_bounds__(256, 2) adj_back_kernel(const AdvanceArgs a, c
 }
 
 // one adjoint kernel: kind 0 forward, 1 backward VJP, 2 replay
-template <int DT, int LAY, int OPT>
+template <int DT, int LAY, int OPT, int SHAPE>
 static const void* adj_kernel(int kind)
 {
     if (kind == 1) return (const void*)adj_back_kernel<DT, LAY, OPT>;
-    if (kind == 2) return (const void*)adj_replay_kernel<DT, LAY, OPT>;
-    return (const void*)adj_forward_kernel<DT, LAY, OPT>;
+    if (kind == 2) return (const void*)adj_replay_kernel<DT, LAY, OPT, SHAPE>;
+    return (const void*)adj_forward_kernel<DT, LAY, OPT, SHAPE>;
+}
+
+template <int LAY, int OPT, int SHAPE>
+static const void* adj_fn_dtype(int kind, int dtype)
+{
+    if (dtype == FTE_BF16) return adj_kernel<FTE_BF16, LAY, OPT, SHAPE>(kind);
+    if (dtype == FTE_F16) return adj_kernel<FTE_F16, LAY, OPT, SHAPE>(kind);
+    return adj_kernel<FTE_F32, LAY, OPT, SHAPE>(kind);
 }
 
 template <int LAY, int OPT>
-static const void* adj_fn_dtype(int kind, int dtype)
+static const void* adj_fn_shape(int kind, int dtype, bool scattered)
 {
-    if (dtype == FTE_BF16) return adj_kernel<FTE_BF16, LAY, OPT>(kind);
-    if (dtype == FTE_F16) return adj_kernel<FTE_F16, LAY, OPT>(kind);
-    return adj_kernel<FTE_F32, LAY, OPT>(kind);
+    return scattered ? adj_fn_dtype<LAY, OPT, kAdjShapeScattered>(kind, dtype)
+                     : adj_fn_dtype<LAY, OPT, kAdjShape>(kind, dtype);
 }
 
 int adjoint_opt(const GridK& g, const ParamsK& prm)
@@ -612,17 +622,18 @@ int adjoint_opt(const GridK& g, const ParamsK& prm)
 }
 
 // record layout and, for the common options (advance_opt: cell records only), the options fixed
-// at compile time, as for the step kernels
-static const void* adj_fn(int kind, int dtype, int pair, int opt)
+// at compile time, as for the step kernels; scattered: see kAdjShape
+static const void* adj_fn(int kind, int dtype, int pair, int opt, bool scattered)
 {
-    if (opt == kOptLinear) return adj_fn_dtype<kLayCell, kOptLinear>(kind, dtype);
-    if (opt == kOptAmrLog) return adj_fn_dtype<kLayCell, kOptAmrLog>(kind, dtype);
-    return pair ? adj_fn_dtype<kLayPair, kOptAny>(kind, dtype) : adj_fn_dtype<kLayCell, kOptAny>(kind, dtype);
+    if (opt == kOptLinear) return adj_fn_dtype<kLayCell, kOptLinear, kAdjShape>(kind, dtype);
+    if (opt == kOptAmrLog) return adj_fn_shape<kLayCell, kOptAmrLog>(kind, dtype, scattered);
+    return pair ? adj_fn_shape<kLayPair, kOptAny>(kind, dtype, scattered)
+                : adj_fn_shape<kLayCell, kOptAny>(kind, dtype, scattered);
 }
 
 cudaError_t adjoint_blocks(int dtype, int pair, int kind, int* blocks_per_sm)
 {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, adj_fn(kind, dtype, pair, kOptAny), 256, 0);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, adj_fn(kind, dtype, pair, kOptAny, false), 256, 0);
 }
 
 static cudaError_t launch_adj(int kind, const AdvanceArgs& a, const AdjK& k, int blocks, cudaStream_t s)
@@ -631,11 +642,16 @@ static cudaError_t launch_adj(int kind, const AdvanceArgs& a, const AdjK& k, int
     const int opt = adjoint_opt(a.g, a.prm);
     // Blocks only decide how warps spread over the SMs, as in launch_advance: one warp per block for
     // a pool that is not reordered (2e4 particles, 400 steps forward and back: 6.32 -> 6.04 ms), 64
-    // threads for a reordered one (2e5 particles x 1024 steps 39.8 -> 38.9 ms).
+    // threads for a reordered one (2e5 particles x 1024 steps 39.8 -> 38.9 ms).  On block AMR a pool
+    // of several waves that is not reordered keeps 256 (2e5 particles, 128 steps forward and back
+    // 16.0 ms with 32, 15.7 with 256; on a uniform grid 10.3 and 10.6).
     const unsigned long long warps = (a.n_particles + 31) / 32, given = (unsigned long long)blocks * 8;
+    const bool scattered = a.g.amr > 0 && !a.order && warps > given;
+    const void* fn = adj_fn(kind, a.g.dtype, a.g.pair, opt, scattered);
+    if (scattered) return cudaLaunchKernel(fn, dim3(blocks), dim3(256), args, 0, s);
     const int nt = a.order ? 64 : 32;
     const unsigned nb = (unsigned)(a.order ? given / 2 : (warps < given ? warps : given));
-    return cudaLaunchKernel(adj_fn(kind, a.g.dtype, a.g.pair, opt), dim3(nb), dim3(nt), args, 0, s);
+    return cudaLaunchKernel(fn, dim3(nb), dim3(nt), args, 0, s);
 }
 
 cudaError_t launch_adjoint_forward(const AdvanceArgs& a, const AdjK& k, int blocks, cudaStream_t s)
