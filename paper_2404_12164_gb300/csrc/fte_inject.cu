@@ -8,19 +8,24 @@
 // of the box, 35 for the slowest of 32), each with a dependent read of a random cell:
 // run one after another per thread, the whole warp waits for its slowest lane
 // (1e6 particles 747 us, and 90-130 us even for a few hundred).  So the warp shares the
-// attempts: every round evaluates one attempt of each particle that has none accepted
-// yet, or 2, 4, .. 32 consecutive attempts of each once at most 16, 8, .. 1 particles are
-// left, and each particle takes its first accepted attempt, which is the one it would
-// have stopped at alone.  The sets of an ensemble go in one launch (each on blocks of its
-// own), and the ledger gets one atomic add per block instead of one per warp: all of them
-// go to the same two addresses.  Measured before -> after: 1e6 particles 747 -> 339 us, 1.2e5
-// 240 -> 68 us, 3.3e4 115 -> 32 us, 64 sets of 4e6 particles together 8.4 -> 1.3 ms.
+// attempts: as long as more than 16 particles have none accepted yet, each makes its own on
+// its lane; once at most 16, 8, .. 1 are left, a round evaluates 2, 4, .. 32 consecutive
+// attempts of each, and each particle takes its first accepted attempt, which is the one
+// it would have stopped at alone.  (With an exchange between the lanes in the rounds of one
+// attempt too, a region where few attempts or none succeed was slower than one thread per
+// particle: 1e6 particles, 100 attempts, none accepted 755 us alone, 1086 with the exchange,
+// 795 as it is; 8 attempts between two looks at the warp, with 1, 4 and 16: 830, 808, 790.)
+// The sets of an ensemble go in one launch (each on blocks of its own), and the ledger gets
+// one atomic add per block instead of one per warp: all of them go to the same two addresses.
+// Measured before -> after: 1e6 particles 747 -> 324 us, 1e5 158 -> 57 us, 3e3 129 -> 35 us, 64
+// sets of 4e6 particles together 8.4 -> 1.3 ms.
 #include "fte_kernels.cuh"
 
 namespace fte {
 
 constexpr int kInjThreads = 256;
 constexpr int kInjWarps = kInjThreads / 32;
+constexpr int kInjAlone = 8;      // attempts of a lane between two looks at the warp
 
 __device__ __forceinline__ double warp_sum_f64(double v)
 {
@@ -37,13 +42,13 @@ __device__ __forceinline__ unsigned warp_sum_u32(unsigned v)
 }
 
 // Position attempt t of particle pid: (r, th, ph), and whether the cell there is accepted.
-__device__ __forceinline__ bool attempt(const GridK& g, const InjectSet& a, float c1, float c2, int t, uint32_t pid,
-                                        uint2 key, float& r, float& th, float& ph)
+// r13, dr3: r1^3 and r2^3 - r1^3; c1, dc: cos(th1) and cos(th2) - cos(th1).
+__device__ __forceinline__ bool attempt(const GridK& g, const InjectSet& a, float r13, float dr3, float c1, float dc,
+                                        int t, uint32_t pid, uint2 key, float& r, float& th, float& ph)
 {
-    const float r13 = a.r1 * a.r1 * a.r1, r23 = a.r2 * a.r2 * a.r2;
     const uint4 q = philox4x32_10(make_uint4((uint32_t)t, pid, 2u, 0u), key);
-    r = cbrtf(r13 + u01(q.x) * (r23 - r13));
-    th = acosf(c1 + u01(q.y) * (c2 - c1));
+    r = cbrtf(r13 + u01(q.x) * dr3);
+    th = acosf(c1 + u01(q.y) * dc);
     ph = a.ph1 + u01(q.z) * (a.ph2 - a.ph1);
     if (a.spiral != 0.f) ph -= a.spiral * (r - a.spiral_rb);   // spiral phase -> longitude
     if (!a.use_divv) return true;
@@ -102,8 +107,8 @@ __global__ void __launch_bounds__(kInjThreads) inject_kernel(const InjectArgs<NS
     }
     const InjectSet& a = k.set[s];
     if (threadIdx.x < 2) {
-        s_c[threadIdx.x] = cosf(threadIdx.x ? a.th2 : a.th1);
-        s_c[2 + threadIdx.x] = powf(threadIdx.x ? a.e2 : a.e1, 1.f - a.gamma);
+        if (a.region == 1) s_c[threadIdx.x] = cosf(threadIdx.x ? a.th2 : a.th1);
+        if (a.energy == 1) s_c[2 + threadIdx.x] = powf(threadIdx.x ? a.e2 : a.e1, 1.f - a.gamma);
     }
     __syncthreads();
     const unsigned long long i = (unsigned long long)(blockIdx.x - a.block0) * kInjThreads + threadIdx.x;
@@ -113,10 +118,16 @@ __global__ void __launch_bounds__(kInjThreads) inject_kernel(const InjectArgs<NS
     float r = a.r, th = a.th, ph = a.ph;
     bool ok = mine;
     if (a.region == 1) {
-        const float c1 = s_c[0], c2 = s_c[1];
+        const float r13 = a.r1 * a.r1 * a.r1, dr3 = a.r2 * a.r2 * a.r2 - r13, c1 = s_c[0], dc = s_c[1] - c1;
         ok = false;
         int t0 = 0;                               // attempts made by every particle still pending
         unsigned pend = __ballot_sync(0xffffffffu, mine);
+        while (__popc(pend) > 16 && t0 < a.max_tries) {
+            const int e = a.max_tries - t0 < kInjAlone ? a.max_tries : t0 + kInjAlone;
+            for (int t = t0; t < e && mine && !ok; ++t) ok = attempt(k.g, a, r13, dr3, c1, dc, t, pid, key, r, th, ph);
+            pend = __ballot_sync(0xffffffffu, mine && !ok);
+            t0 = e;
+        }
         while (pend != 0u && t0 < a.max_tries) {
             const int u = __popc(pend);
             const AttemptRound round(u, t0, a.max_tries);
@@ -132,7 +143,7 @@ __global__ void __launch_bounds__(kInjThreads) inject_kernel(const InjectArgs<NS
             const uint32_t opid = pid - lane + owner;     // ids are consecutive within the warp
             float tr = 0.f, tth = 0.f, tph = 0.f;
             bool hit = false;
-            if (works) hit = attempt(k.g, a, c1, c2, t0 + j, opid, key, tr, tth, tph);
+            if (works) hit = attempt(k.g, a, r13, dr3, c1, dc, t0 + j, opid, key, tr, tth, tph);
             const unsigned hits = __ballot_sync(0xffffffffu, hit);
             const unsigned seg = waits ? (hits >> (rank * g)) & (g == 32 ? 0xffffffffu : (1u << g) - 1u) : 0u;
             // the accepted attempt, or the last one of a particle that runs out of attempts

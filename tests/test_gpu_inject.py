@@ -93,3 +93,22 @@ def test_refused_set_keeps_the_sets_before_it(cir):
     with pytest.raises(Exception):
         api.fte_inject_batched(pool, bg, [good, bad], tally)
     assert pool.count == 40 and api.fte_ledger(tally)[1][0] + api.fte_ledger(tally)[1][5] == 40
+
+
+@pytest.mark.parametrize("max_tries", [7, 8, 9, 17, 40])
+@pytest.mark.parametrize("n", [16, 17, 600])
+def test_rare_positions(cir, n, max_tries):
+    """Few attempts succeed, so that most of a warp stays pending: the attempts that lanes make alone
+    end at the limit whether or not it is a multiple of the number between two votes (of 600, the
+    oracle gives up on 86 % after 40 attempts and on 98 % after 7)."""
+    from paper_2404_12164_gb300 import api
+    w, bg, obg = cir
+    spec = dataclasses.replace(w.inject, max_tries=max_tries, seed=7 * n + max_tries, divv_max=-1e-5)
+    pool, tally = api.Particles(n), api.Tally([])
+    api.fte_inject(pool, bg, spec, n, tally, check_failed=False)
+    ref, _ = O.inject(obg, spec, np.arange(n))
+    st = pool.state()
+    _compare(st, ref)
+    assert (st["status"] == O.INJ_FAIL).sum() == api.fte_ledger(tally)[1][5]
+    if n == 600:
+        assert 0.8 * n < (st["status"] == O.INJ_FAIL).sum() < n
