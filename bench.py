@@ -291,6 +291,23 @@ def e2e_breakdown(api, pool, ring_bg, sstream, w, tally, wsp, id_base, stream, b
 # ---------------------------------------------------------------------------
 # GPU arm
 # ---------------------------------------------------------------------------
+def kernel_launches(n_part, n_steps, sort_every, tally_layout, sms):
+    """The library's kernels of one timed step: tally reset and inject, and per advance call the
+    normalisation's partial sums and the set-up (its final sums and the step table), then per launch
+    chunk the step kernel, (with the shared-memory tally) the reduction of the counts and (with
+    reordering) the key, scan and scatter kernels and, from a call's second chunk on, the clear.  A
+    reordered pool of at least one wave of the step kernel's threads (512 per SM) with the global
+    tally is advanced as two halves, each with its own reordering and launches."""
+    halves = 2 if sort_every > 0 and tally_layout == "global" and n_part >= 512 * sms else 1
+    chunk = min(sort_every, 1024) if sort_every > 0 else 1024      # steps of a launch
+    total = 2
+    for c in range(0, n_steps, CHUNK):
+        chunks = math.ceil(min(CHUNK, n_steps - c) / chunk)
+        per_half = chunks * (1 + (tally_layout == "shared")) + (4 * chunks - 1 if sort_every > 0 else 0)
+        total += 2 + per_half * halves
+    return total
+
+
 def run_gpu(args):
     import torch
     import torch.distributed as dist
@@ -458,22 +475,8 @@ def run_gpu(args):
                                                                           adjoint["t_c"]))
 
     roofline = roofline_record(intervals, total_steps // ws, ALG_BYTES, l1, l2_gbs, measured_traffic(args.layout))
-    # our kernels per timed step: tally reset and inject, and per advance call the normalisation's
-    # partial sums and the set-up (its final sums and the step table), then per launch chunk the
-    # step kernel, (with the shared-memory tally) the partial-histogram reduction and (with
-    # reordering) the key, scan and scatter kernels and, from a call's second chunk on, the clear
-    # a pool of at least one wave of threads (at most 3 blocks of 256 per SM) is advanced as
-    # two halves, each with its own reordering and launches (global tally, reordering on)
-    wave = torch.cuda.get_device_properties(local).multi_processor_count * 3 * 256
-    halves = 2 if (w.params.sort_every > 0 and w.params.tally_layout == "global" and n_part >= wave) else 1
-
-    def kernels_per_call(s):
-        chunk = min(w.params.sort_every, CHUNK) if w.params.sort_every > 0 else CHUNK
-        chunks = math.ceil(s / chunk)
-        per_chunk = 1 + (1 if w.params.tally_layout == "shared" else 0)
-        sort = 4 * chunks - 1 if w.params.sort_every > 0 else 0
-        return 2 + (chunks * per_chunk + sort) * halves
-    launches_per_step = 2 + sum(kernels_per_call(min(CHUNK, n_steps - c)) for c in range(0, n_steps, CHUNK))
+    launches_per_step = kernel_launches(n_part, n_steps, w.params.sort_every, w.params.tally_layout,
+                                        torch.cuda.get_device_properties(local).multi_processor_count)
     result = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,

@@ -83,3 +83,16 @@ def test_ring_upload_count():
     frozen = [(i * 60, (i + 1) * 60, i) for i in range(5)] + [(300, 800, -1 - 5)]
     for R in (2, 3, 6):
         assert bench.ring_uploads(frozen, R, 6, False) == 6
+
+
+def test_kernel_launches_counts_the_halves_of_one_wave():
+    """A pool is split from one wave of 512 threads per SM on, whatever lies between that and 768."""
+    sms = 152
+    # reset, inject, 2 set-up kernels, and per 64-step chunk key, scan, scatter, step, and 15 clears
+    one = 2 + 2 + 16 * 4 + 15
+    assert bench.kernel_launches(512 * sms - 1, 1024, 64, "global", sms) == one
+    for n in (512 * sms, 600 * sms, 767 * sms, 10 ** 6):
+        assert bench.kernel_launches(n, 1024, 64, "global", sms) == 4 + 2 * (one - 4)
+    assert bench.kernel_launches(10 ** 6, 1024, 64, "shared", sms) == one + 16
+    assert bench.kernel_launches(10 ** 6, 1024, 0, "global", sms) == 5
+    assert bench.kernel_launches(10 ** 6, 2 * 1024 + 1, 0, "global", sms) == 4 + 3
