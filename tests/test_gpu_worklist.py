@@ -57,3 +57,25 @@ def test_every_particle_once(parker, n, sort):
     assert np.array_equal(ledger, rledger)
     assert ledger[6] == n * STEPS            # nothing leaves the domain from 1 au in 200 s
     assert np.array_equal(counts, rcounts)
+
+
+@pytest.mark.parametrize("per_sm,more", [(32, -1), (32, 0), (32, 1), (64, 1), (512, -1), (512, 0), (512, 1)])
+@pytest.mark.parametrize("sort", [0, 8])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_every_particle_once_at_this_device_s_edges(parker, per_sm, more, sort, dtype):
+    """Ranges of exactly one and two batches and one wave, by this device's number of SMs; 16-bit
+    pools, which take their work from one counter, too."""
+    import torch
+    from paper_2404_12164_gb300 import api
+    w, bg = parker
+    if dtype != "f32":
+        img = api.Background(w.grid, dtype=dtype)
+        api.fte_quantize_background(img, bg)
+        bg = img
+    n = torch.cuda.get_device_properties(0).multi_processor_count * per_sm + more
+    st, ledger, counts = _run(w, bg, n, sort, False)
+    ref, rledger, rcounts = _run(w, bg, n, 0, True)
+    for k in ref:
+        assert np.array_equal(st[k], ref[k]), k
+    assert np.array_equal(ledger, rledger) and ledger[6] == n * STEPS
+    assert np.array_equal(counts, rcounts)
