@@ -139,8 +139,8 @@ cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, 
     // spread over the SMs.  A pool that is not reordered goes in blocks of one warp: 1e4 particles
     // in blocks of 256 occupy 40 of 152 SMs with 8 warps each, in blocks of 32 every SM with 2, and
     // a step's latency falls with the warps it shares an SM with (1e4 particles x 8640 steps 19.1
-    // -> 17.4 ms, 2000 x 200 0.54 -> 0.50 ms); 1.3e5 particles, two per thread, are 248 blocks of
-    // 256, two on 96 SMs and one on 56.  A reordered pool launches one wave in blocks of 64: when
+    // -> 17.4 ms, 2000 x 200 0.54 -> 0.50 ms); 1.3e5 particles, two per thread, are 254 blocks of
+    // 256, two on 102 SMs and one on 50.  A reordered pool launches one wave in blocks of 64: when
     // few particles are left alive and the surplus blocks leave at once (see advance_kernel), those
     // that stay are spread as evenly (1e6 particles over 4 days, 4.6e4 alive at the end: 543 ms in
     // blocks of 256, 531 of 128, 530 of 64, 528 of 32; 1.2e5 with cross-field diffusion 929 -> 910
