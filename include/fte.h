@@ -291,8 +291,8 @@ size_t fte_tally_bins(const fte_tally_buf* t);
 fte_status fte_tally_reset(const fte_tally_buf* t, void* stream);
 
 /* Scratch (DEVICE) needed by fte_advance on `device` for grid `g`, tally `t`, a
-   pool of `n_particles` entries and `n_steps` steps per call: per-block partial
-   histograms, launch counters, the per-step time table, the normalisation
+   pool of `n_particles` entries and `n_steps` steps per call: per-block step
+   counts, launch counters, the per-step time table, the normalisation
    constants and the particle-ordering buffers.  0 on error. */
 size_t fte_workspace_bytes(int device, const fte_grid* g, const fte_tally_buf* t,
                            uint64_t n_particles, int64_t n_steps);
@@ -415,8 +415,8 @@ fte_status fte_stream_load(const fte_background* bg, const void* host_snapshots,
    cudaDeviceReset (or any teardown of that context) invalidates it, after which
    the process must not call this entry point on that device again.  All calls
    share the array: calls whose work overlaps on the GPU race on it.  Returns
-   FTE_ENOMEM when the tally's per-block partial histograms (12 bytes per bin) do
-   not fit the array for at least one block per SM (about 13,800 bins on a
+   FTE_ENOMEM when 12 bytes per bin and block (of which the counts use 4) do not
+   fit the array for at least one block per SM (about 13,800 bins on a
    152-SM GB300). */
 fte_status fte_advance_noalloc(fte_particles* P, const fte_background* bg, const fte_params* prm,
                                const fte_tally_buf* t, int64_t n_start, int64_t n_end, void* stream);

@@ -8,7 +8,8 @@ namespace fte {
 // single-set kernels without cross-field diffusion are compiled for exactly the two blocks of
 // 256 threads per SM that they get: told so, the compiler uses all 128 registers and keeps more
 // record loads in flight (left to itself it took 104 - 110; 1e6 particles over 4 days of
-// snapshots 603 -> 577 ms, 1e4 Parker particles 14.8 -> 13.2 ms).  The cross-field builds use
+// snapshots 603 -> 577 ms, 1e4 Parker particles 14.8 -> 13.2 ms; 28 - 56 bytes of spills, about
+// one spilled load per step of 876 instructions).  The cross-field builds use
 // 128 anyway and measured 2 % faster left alone.
 constexpr int kMinBlocks = 512 / kThreads;
 
@@ -47,7 +48,8 @@ static const void* dense_fn(int dtype)
     return (const void*)advance_kernel<false, FTE_F32, kModeSingleGlobal, kAmr32Threads, LAY, kAmr32Blocks, OPT, SHAPE>;
 }
 
-// FP32 records, 5 blocks of 128 threads, 20 warps per SM at 102 registers (see advance_opt)
+// FP32 records, 5 blocks of 128 threads, 20 warps per SM at 96 registers, 64 - 80 bytes of spills
+// (see advance_opt)
 template <int LAY>
 static const void* warps_fn()
 {
@@ -144,7 +146,7 @@ cudaError_t launch_advance(const AdvanceArgs& a, const BatchArgs& b, int kperp, 
     // few particles are left alive and the surplus blocks leave at once (see advance_kernel), those
     // that stay are spread as evenly (1e6 particles over 4 days, 4.6e4 alive at the end: 543 ms in
     // blocks of 256, 531 of 128, 530 of 64, 528 of 32; 1.2e5 with cross-field diffusion 929 -> 910
-    // us).  A block of the shared-memory tally carries a whole histogram and stays as it is.
+    // us).  A block of the shared-memory tally carries a count of every bin and stays as it is.
     if (mode == kModeSingleGlobal) {
         const int small = a.order ? 64 : 32;
         const unsigned long long need = (a.n_particles + small - 1) / small,

@@ -613,7 +613,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
     if (s != FTE_OK) return s;
     if (prm && prm->tally_layout != 0 && prm->tally_layout != FTE_LAYOUT_SHARED && prm->tally_layout != FTE_LAYOUT_GLOBAL)
         return fail(FTE_EINVAL, "bad tally layout");
-    // the warp-merged FP64 atomics unless the shared-memory histogram is asked for
+    // every accumulator by atomics in global memory unless counts in shared memory are asked for
     const int mode = (prm && prm->tally_layout == FTE_LAYOUT_SHARED) ? kModeSingle : kModeSingleGlobal;
     if (mode == kModeSingle && nb > (size_t)kMaxSmemBins)
         return fail(FTE_ENOTSUP, "%zu tally bins exceed %d", nb, kMaxSmemBins);
@@ -712,7 +712,7 @@ fte_status fte_advance(fte_particles* P, const fte_background* bg, const fte_par
     // Two halves on two streams: while the last particles of one half's launch run, the
     // other half's reordering and launch fill the idle SMs (the step kernel launches one
     // wave of persistent blocks and its end waits for its slowest thread).  Only with the
-    // global tally (no per-block partials), a pool of at least one wave, and outside
+    // global tally (no per-block counts), a pool of at least one wave, and outside
     // stream capture; each particle's result does not depend on it.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     FTE_CUDA(cudaStreamIsCapturing(st, &cap), "capture query");
@@ -996,7 +996,7 @@ extern "C" fte_status fte_advance_noalloc(fte_particles* P, const fte_background
     if (prm->dmumu == 0 && !(prm->q > 1.0 && prm->q <= 2.0 && prm->H >= 0.0)) return fail(FTE_EINVAL, "need 1 < q <= 2, H >= 0");
     if (prm->dmumu == 1 && !(prm->eps > 0.0)) return fail(FTE_EINVAL, "eps must be > 0");
     if (prm->lambda_perp < 0.0) return fail(FTE_EINVAL, "lambda_perp must be >= 0");
-    // the tally always goes through per-block shared-memory histograms here; other layout
+    // the steps are always counted in shared memory here; other layout
     // values are refused as fte_advance refuses them
     if (prm->tally_layout != 0 && prm->tally_layout != FTE_LAYOUT_SHARED && prm->tally_layout != FTE_LAYOUT_GLOBAL)
         return fail(FTE_EINVAL, "bad tally_layout %d", prm->tally_layout);

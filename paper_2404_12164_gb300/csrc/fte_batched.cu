@@ -1,6 +1,6 @@
 // Ensemble variants of the step kernel (many parameter sets in one launch):
-// per-set tallies either in shared memory (all sets' bins per block) or merged
-// per warp into FP64 accumulators in global memory, at 128 or 256 threads per
+// per-set tallies in FP64 accumulators in global memory, their counts there too or per
+// block in shared memory (all sets' bins), at 128 or 256 threads per
 // block, for the cell or the pair record layout (compile-time, as for the
 // single-set kernels).  The step arithmetic is the single-set kernel's (fte_step.cuh).
 #include "fte_step.cuh"
